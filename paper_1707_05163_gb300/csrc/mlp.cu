@@ -229,50 +229,100 @@ __global__ void gelu_backward(const float *dact, const __nv_bfloat16 *pre, int64
   }
 }
 
-// column sums of an FP32 [M x N] matrix: one thread per column, fixed order
-__global__ void column_sums(const float *x, int64_t M, int N, float *out) {
+// Column sums of an FP32 [M x N] matrix (N a multiple of 64), in two stages
+// of fixed order: block (x, y) sums the rows [x * rows, (x + 1) * rows) of the
+// 64 columns of group y -- 16 lanes of four columns side by side, 16 rows at a
+// time, then the 16 row lanes in order -- into part[x][N].  Bound by the read
+// of the matrix (16 MB at 16384 x 256: 5 us); one thread per column over all
+// rows, as it was, is a chain of M dependent additions (550 us).
+constexpr int kColThreads = 256;
+__global__ void __launch_bounds__(kColThreads) column_sums_part(const float *x, int64_t M, int N,
+                                                                int64_t rows, float *part) {
+  __shared__ float4 sh[16][16];
+  const int lc = threadIdx.x & 15, lr = threadIdx.x >> 4;
+  const int c0 = blockIdx.y * 64 + lc * 4;
+  const int64_t r0 = (int64_t)blockIdx.x * rows;
+  const int64_t r1 = r0 + rows < M ? r0 + rows : M;
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+  for (int64_t r = r0 + lr; r < r1; r += 16) {
+    const float4 v = *reinterpret_cast<const float4 *>(x + r * N + c0);
+    s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+  }
+  sh[lr][lc] = s;
+  __syncthreads();
+  if (lr == 0) {
+#pragma unroll
+    for (int q = 1; q < 16; ++q) {
+      const float4 v = sh[q][lc];
+      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+    }
+    *reinterpret_cast<float4 *>(part + (size_t)blockIdx.x * N + c0) = s;
+  }
+}
+__global__ void column_sums_final(const float *part, int nparts, int N, float *out) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= N) return;
   float s = 0.f;
-  for (int64_t r = 0; r < M; ++r) s += x[r * N + c];
+#pragma unroll 8
+  for (int p = 0; p < nparts; ++p) s += part[(size_t)p * N + c];
   out[c] = s;
 }
 
-// BF16 [M x N] -> FP32 copy
-__global__ void bf16_to_f32(const __nv_bfloat16 *x, int64_t n, float *y) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    y[i] = __bfloat162float(x[i]);
+// Eight values as BF16 in one 16-byte store (dst 16-byte aligned).
+__device__ __forceinline__ void store_bf16x8(__nv_bfloat16 *dst, const float (&v)[8]) {
+  uint32_t w[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+    w[j] = *reinterpret_cast<const uint32_t *>(&h);
+  }
+  *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// FP32 [M x n_real] features -> BF16 [M x ld] zero-padded
+// FP32 [M x n_real] features -> BF16 [M x ld] zero-padded, eight columns per
+// thread (ld a multiple of 64)
 __global__ void pack_input(const float *x, int64_t M, int n_real, int ld, __nv_bfloat16 *out) {
-  const int64_t total = M * ld;
+  const int cpr = ld / 8;
+  const int64_t total = M * cpr;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / ld;
-    const int c = (int)(i - r * ld);
-    out[i] = __float2bfloat16_rn(c < n_real ? x[r * n_real + c] : 0.f);
+    const int64_t r = i / cpr;
+    const int c = (int)(i - r * cpr) * 8;
+    float v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = c + j < n_real ? x[r * n_real + c + j] : 0.f;
+    store_bf16x8(out + r * ld + c, v);
   }
 }
 
 // MSE loss 0.5 * mean over rows of sum over the n_out outputs of (y - t)^2
-// with output gradient (y - t) / M (FP32, padded columns zero).
+// with output gradient (y - t) / M in FP32 and BF16 (padded columns zero),
+// eight columns per thread (ldy a multiple of 64).
 __global__ void mse_grad(const float *y, int ldy, const float *t, int n_out, int64_t M,
-                         float *dy, float *loss_partial) {
+                         float *dy, __nv_bfloat16 *dyb, float *loss_partial) {
   __shared__ float sh[256];
+  const int cpr = ldy / 8;
+  const int64_t total = M * cpr;
   float l = 0.f;
-  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < M;
-       r += (int64_t)gridDim.x * blockDim.x) {
-    for (int c = 0; c < ldy; ++c) {
-      float g = 0.f;
-      if (c < n_out) {
-        const float d = y[r * ldy + c] - t[r * n_out + c];
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = i / cpr;
+    const int c0 = (int)(i - r * cpr) * 8;
+    float g[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      g[j] = 0.f;
+      if (c0 + j < n_out) {
+        const float d = y[r * ldy + c0 + j] - t[r * n_out + c0 + j];
         l += 0.5f * d * d;
-        g = d / (float)M;
+        g[j] = d / (float)M;
       }
-      dy[r * ldy + c] = g;
     }
+    float4 *d4 = reinterpret_cast<float4 *>(dy + r * ldy + c0);
+    d4[0] = make_float4(g[0], g[1], g[2], g[3]);
+    d4[1] = make_float4(g[4], g[5], g[6], g[7]);
+    store_bf16x8(dyb + r * ldy + c0, g);
   }
   sh[threadIdx.x] = l;
   __syncthreads();
@@ -363,6 +413,8 @@ struct pg_mlp {
   float *gscratch = nullptr;          // split-K partials of the weight gradient
   size_t gscratch_bytes = 0;
   float *loss_partial = nullptr;
+  float *colpart = nullptr;           // column-sum partials of the bias gradients
+  int col_rows = 0;                   // its rows: at most this many partials
   int use_tc = 0;                     // tcgen05 products when available
   int fused = 1;                      // tcgen05 inference in one fused kernel when the shape allows
   uint8_t *wpk = nullptr;             // weights packed for the fused forward
@@ -374,7 +426,9 @@ namespace pg {
 cudaError_t gemm_nt_tc(const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, int ldb,
                        int64_t M, int N, int K, const float *bias, int act, float *out_f32,
                        __nv_bfloat16 *out_bf16, __nv_bfloat16 *pre_bf16, int ldc, cudaStream_t st,
-                       int *err, const __nv_bfloat16 *gin = nullptr);
+                       int *err, const __nv_bfloat16 *gin = nullptr, float *colpart = nullptr,
+                       int *nparts = nullptr);
+int gemm_tc_max_ctas();
 size_t mlp_fused_packed_bytes();
 cudaError_t mlp_fused_pack(const __nv_bfloat16 *const w[5], uint8_t *out, cudaStream_t st);
 cudaError_t mlp_fused_forward(const float *x, int64_t M, int n_in, const uint8_t *wpk,
@@ -385,7 +439,8 @@ cudaError_t mlp_fused_step_launch(const SurrogateStepIO &io, const uint8_t *wpk,
 cudaError_t mlp_wait_probe(long long polls, int *err, cudaStream_t st);
 cudaError_t gemm_tn_splitk_tc(const __nv_bfloat16 *A, int64_t lda, int Mrows,
                               const __nv_bfloat16 *B, int64_t ldb, int N, int64_t K, float *out,
-                              float *scratch, size_t scratch_bytes, cudaStream_t st, int *err);
+                              float *scratch, size_t scratch_bytes, const float *bpart, int nparts,
+                              float *bout, cudaStream_t st, int *err);
 }
 
 namespace {
@@ -399,7 +454,8 @@ void free_ws(pg_mlp *n) {
   dev_free(n->y); dev_free(n->dy); dev_free(n->dyb); dev_free(n->dyt); dev_free(n->xt);
   dev_free(n->dyb2); dev_free(n->gscratch);
   n->dyb2 = nullptr; n->gscratch = nullptr; n->gscratch_bytes = 0;
-  dev_free(n->loss_partial);
+  dev_free(n->loss_partial); dev_free(n->colpart);
+  n->colpart = nullptr;
   n->x0 = nullptr; n->y = nullptr; n->dy = nullptr; n->dyb = nullptr; n->dyt = nullptr;
   n->xt = nullptr; n->loss_partial = nullptr;
   n->cap = 0;
@@ -432,6 +488,8 @@ cudaError_t ensure_ws(pg_mlp *n, int64_t rows) {
   al((void **)&n->dyt, cap * wmax * 2);
   al((void **)&n->xt, cap * std::max(n->width, n->pin) * 2);
   al((void **)&n->loss_partial, 1024 * 4);
+  n->col_rows = std::max(gemm_tc_max_ctas(), 128);
+  al((void **)&n->colpart, (size_t)n->col_rows * wmax * 4);
   if (e != cudaSuccess) {
     free_ws(n);
     return e;
@@ -484,40 +542,56 @@ cudaError_t forward(pg_mlp *n, int64_t rows, cudaStream_t st, bool keep) {
   return cudaSuccess;
 }
 
-// backward from n->dy (gradient of the FP32 output, [rows x pout]) into n->g
+// backward from n->dy and n->dyb (gradient of the output in FP32 and BF16,
+// [rows x pout]) into n->g, which it writes whole
 cudaError_t backward(pg_mlp *n, int64_t rows, cudaStream_t st) {
   cudaError_t e;
-  // gradient w.r.t. the current layer's pre-activation (BF16 copy in dyb)
-  int wcur = n->pout;
-  f32_to_bf16<<<grid1(rows * wcur), 256, 0, st>>>(n->dy, rows * wcur, n->dyb);
-  note_launches(1);
+  bool have_part = false;      // colpart holds the sums of the current gradient
+  int nparts = 0;
   for (int l = n->nl - 1; l >= 0; --l) {
     const __nv_bfloat16 *X = l == 0 ? n->x0 : n->act[l - 1];
     const int din = n->din[l], dout = n->dout[l];
-    // bias gradient: column sums of dPre (FP32, in dy)
-    column_sums<<<(dout + 127) / 128, 128, 0, st>>>(n->dy, rows, dout, n->g + n->boff[l]);
-    // dW [dout x din] = dPre^T X: transposes to K-contiguous [dout x rows], [din x rows]
-    dim3 g1((dout + 31) / 32, (unsigned)((rows + 31) / 32));
-    transpose_bf16<<<g1, dim3(32, 8), 0, st>>>(n->dyb, (int)rows, dout, dout, n->dyt, (int)rows);
-    dim3 g2((din + 31) / 32, (unsigned)((rows + 31) / 32));
-    transpose_bf16<<<g2, dim3(32, 8), 0, st>>>(X, (int)rows, din, din, n->xt, (int)rows);
-    note_launches(3);
     const bool tc = n->use_tc && (din == 64 || din == 256) && (dout == 64 || dout == 256);
-    // rows must be a multiple of 32 for the K loop; the batch is padded
-    if (tc) e = gemm_tn_splitk_tc(n->dyt, rows, dout, n->xt, rows, din, rows, n->g + n->woff[l],
-                                  n->gscratch, n->gscratch_bytes, st, n->d_err);
-    else e = gemm_nt(n->dyt, (int)rows, n->xt, (int)rows, dout, din, (int)rows, nullptr, 0,
-                     n->g + n->woff[l], nullptr, nullptr, din, 0, st);
+    // bias gradient: column sums of dPre in FP32, from the product that made
+    // it or, where that kept no sums, from dy
+    if (!have_part) {
+      const int64_t per = std::max<int64_t>(64, ((rows + 127) / 128 + 15) / 16 * 16);
+      nparts = (int)((rows + per - 1) / per);
+      column_sums_part<<<dim3((unsigned)nparts, (unsigned)(dout / 64)), kColThreads, 0, st>>>(
+          n->dy, rows, dout, per, n->colpart);
+      note_launches(1);
+    }
+    // dW [dout x din] = dPre^T X
+    if (tc) {
+      e = gemm_tn_splitk_tc(n->dyb, dout, dout, X, din, din, rows, n->g + n->woff[l], n->gscratch,
+                            n->gscratch_bytes, n->colpart, nparts, n->g + n->boff[l], st, n->d_err);
+    } else {
+      column_sums_final<<<(dout + 127) / 128, 128, 0, st>>>(n->colpart, nparts, dout,
+                                                            n->g + n->boff[l]);
+      // transposes to K-contiguous [dout x rows], [din x rows]
+      dim3 g1((dout + 31) / 32, (unsigned)((rows + 31) / 32));
+      transpose_bf16<<<g1, dim3(32, 8), 0, st>>>(n->dyb, (int)rows, dout, dout, n->dyt, (int)rows);
+      dim3 g2((din + 31) / 32, (unsigned)((rows + 31) / 32));
+      transpose_bf16<<<g2, dim3(32, 8), 0, st>>>(X, (int)rows, din, din, n->xt, (int)rows);
+      note_launches(3);
+      // rows must be a multiple of 32 for the K loop; the batch is padded
+      e = gemm_nt(n->dyt, (int)rows, n->xt, (int)rows, dout, din, (int)rows, nullptr, 0,
+                  n->g + n->woff[l], nullptr, nullptr, din, 0, st);
+    }
     if (e != cudaSuccess) return e;
     if (l == 0) break;
     if (tc) {
       // dPre of layer l-1 = (dPre W) * GELU'(pre) in one product (B = W^T
-      // [din x dout]); FP32 into dy, BF16 into the other buffer (the one
-      // read as A must not be overwritten by other tiles)
+      // [din x dout]), in BF16 into the other buffer (the one read as A must
+      // not be overwritten by other tiles), with its column sums; in FP32 only
+      // for a next layer that goes the other way
+      const int dn = n->din[l - 1];
+      const bool tc_next = (dn == 64 || dn == 256) && (din == 64 || din == 256);
       if ((e = gemm_nt_tc(n->dyb, dout, n->wbt + n->woff[l], dout, rows, din, dout, nullptr, 2,
-                          n->dy, n->dyb2, nullptr, din, st, n->d_err, n->pre[l - 1])) !=
-          cudaSuccess)
+                          tc_next ? nullptr : n->dy, n->dyb2, nullptr, din, st, n->d_err,
+                          n->pre[l - 1], n->colpart, &nparts)) != cudaSuccess)
         return e;
+      have_part = true;
       std::swap(n->dyb, n->dyb2);
     } else {
       // dX [rows x din] = dPre W  (B = W^T [din x dout])
@@ -528,8 +602,8 @@ cudaError_t backward(pg_mlp *n, int64_t rows, cudaStream_t st) {
       gelu_backward<<<grid1(rows * din), 256, 0, st>>>(n->dy, n->pre[l - 1], rows, din, n->dyb,
                                                        n->dy);
       note_launches(1);
+      have_part = false;
     }
-    wcur = din;
   }
   return cudaGetLastError();
 }
@@ -722,7 +796,7 @@ pg_status pg_mlp_forward(pg_mlp *n, const float *x, int64_t M, float *y, void *s
   for (int64_t r0 = 0; r0 < M && !fused; r0 += chunk) {
     const int64_t rows = std::min(chunk, M - r0);
     CUM(ensure_ws(n, std::min<int64_t>(M, chunk)));
-    pack_input<<<grid1(rows * n->pin), 256, 0, st>>>(x + r0 * n->n_in, rows, n->n_in, n->pin, n->x0);
+    pack_input<<<grid1(rows * (n->pin / 8)), 256, 0, st>>>(x + r0 * n->n_in, rows, n->n_in, n->pin, n->x0);
     note_launches(1);
     CUM(forward(n, rows, st, false));
     CUM(cudaMemcpy2DAsync(y + r0 * n->n_out, n->n_out * 4, n->y, n->pout * 4, n->n_out * 4, rows,
@@ -748,13 +822,12 @@ static pg_status mlp_grad_impl(pg_mlp *n, const float *x, const float *t, int64_
                                cudaStream_t st) {
   if (M % 32) { set_error("invalid argument: batch size must be a multiple of 32"); return PG_ERR_ARG; }
   CUM(ensure_ws(n, M));
-  pack_input<<<grid1(M * n->pin), 256, 0, st>>>(x, M, n->n_in, n->pin, n->x0);
+  pack_input<<<grid1(M * (n->pin / 8)), 256, 0, st>>>(x, M, n->n_in, n->pin, n->x0);
   note_launches(1);
   CUM(forward(n, M, st, true));
-  const int nb = (int)std::min<int64_t>(1024, (M + 255) / 256);
-  mse_grad<<<nb, 256, 0, st>>>(n->y, n->pout, t, n->n_out, M, n->dy, n->loss_partial);
+  const int nb = (int)std::min<int64_t>(1024, (M * (n->pout / 8) + 255) / 256);
+  mse_grad<<<nb, 256, 0, st>>>(n->y, n->pout, t, n->n_out, M, n->dy, n->dyb, n->loss_partial);
   note_launches(1);
-  CUM(cudaMemsetAsync(n->g, 0, n->nparam * 4, st));
   CUM(backward(n, M, st));
   if (n->use_tc) {
     int err = 0;

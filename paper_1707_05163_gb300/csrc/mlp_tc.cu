@@ -4,15 +4,19 @@
 // BF16 operands, FP32 accumulation in tensor memory (TMEM), N and K in {64,
 // 256}; act 1 applies GELU, act 2 multiplies by GELU'(g) of a stored
 // pre-activation g (the input gradient through the activation).  Weight
-// gradient: a split-K product D[M x N] = A[M x K] . B[N x K]^T with K the
+// gradient: a split-K product D[M x N] = A[K x M]^T . B[K x N] with K the
 // batch (gemm_tn_splitk_tc below).  Persistent
 // CTAs (one per SM): each loads B once into shared memory and then walks
 // 128-row tiles of A.  Per tile: one thread issues K/16 tcgen05.mma (128 x N
 // x 16) on the A tile in shared memory and commits them to an mbarrier, all
 // threads wait on it (bounded), start copying the next A tile into the now
-// free buffer (cp.async), and meanwhile each warp reads its 32 accumulator
-// rows from TMEM (tcgen05.ld) and applies bias, GELU and the BF16/FP32
-// stores.
+// free buffer (cp.async), and meanwhile each warp reads a 16-column piece
+// of its lane group's 32 accumulator rows from TMEM (tcgen05.ld) and applies
+// bias, GELU and the BF16/FP32 stores; sixteen warps, four per lane group,
+// because the piece loop is a chain of waits (tensor memory, the stored
+// pre-activation).  A gradient of 16384 rows of the surrogate network took
+// 3154 us with serial column sums, ten transposed copies and four-warp
+// epilogues, and takes 339 us.
 //
 // Shared-memory operand layout (K-major, no swizzle): 8-row x 16-byte core
 // matrices; core matrix (row group g, 16-byte K chunk c) sits at byte
@@ -30,7 +34,9 @@ namespace pg {
 namespace {
 
 constexpr int TM = 128;
-constexpr int kTcThreads = 128;
+constexpr int kTcThreads = 512;
+constexpr int kTcWarps = kTcThreads / 32;
+constexpr int kColGroups = kTcWarps / 4;     // warps that share a lane group split the columns
 constexpr long long kSpinLimit = 20000000;   // mbarrier polls before giving up
 
 __device__ __forceinline__ uint32_t su32(const void *p) {
@@ -88,15 +94,37 @@ __device__ __forceinline__ void store_bf16x16(__nv_bfloat16 *dst, const float (&
   reinterpret_cast<uint4 *>(dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
 }
 
+// Sums over the warp's 32 lanes of 16 values per lane: a reduce-scatter of 16
+// shuffles (five per value as 16 separate sums would be 80).  Lane l returns
+// the sum of column col(l) = 8 b4 + 4 b3 + 2 b2 + b1 (the bits of l); v is
+// used up.  Fixed order, so the result does not depend on timing.
+__device__ __forceinline__ float warp_column_sums16(float (&v)[16], int lane) {
+#pragma unroll
+  for (int w = 8, bit = 16; w >= 1; w >>= 1, bit >>= 1) {
+    const bool up = (lane & bit) != 0;
+#pragma unroll
+    for (int j = 0; j < w; ++j) {
+      const float keep = up ? v[j + w] : v[j], send = up ? v[j] : v[j + w];
+      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+    }
+  }
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
 // copy rows [0, rows) of a K-wide BF16 matrix (row stride ld) into the
-// core-matrix layout; rows in [rows, R) are zero-filled
+// core-matrix layout; rows in [rows, R) are zero-filled (R a multiple of 8).
+// Eight lanes take the eight rows of a core matrix, 128 contiguous bytes of
+// shared memory, and the warp four neighbouring chunks, 64 bytes of each row.
+// (Lanes along a row would write at a stride of 128 bytes, all to the same
+// banks: 6 us of a 256 x 256 product's 23.)
 template <int K>
 __device__ __forceinline__ void load_tile(uint8_t *dst, const __nv_bfloat16 *src, int ld, int rows,
                                           int R) {
   constexpr int KC = K / 8;   // 16-byte chunks per row
   for (int idx = threadIdx.x; idx < R * KC; idx += kTcThreads) {
-    const int r = idx / KC, c = idx - r * KC;
-    const uint32_t off = (uint32_t)(((r >> 3) * KC + c) * 128 + (r & 7) * 16);
+    const int r8 = idx & 7, c = (idx >> 3) % KC, g = (idx >> 3) / KC;
+    const int r = g * 8 + r8;
+    const uint32_t off = (uint32_t)((g * KC + c) * 128 + r8 * 16);
     const bool ok = r < rows;
     const __nv_bfloat16 *s = src + (size_t)(ok ? r : 0) * ld + c * 8;
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(su32(dst + off)),
@@ -124,7 +152,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 gemm_tc_kernel(const __nv_bfloat16 *__restrict__ A, int lda, const __nv_bfloat16 *__restrict__ B,
                int ldb, int64_t M, const float *__restrict__ bias, int act, float *out_f32,
                __nv_bfloat16 *out_bf16, __nv_bfloat16 *pre_bf16,
-               const __nv_bfloat16 *__restrict__ gin, int ldc, int *err) {
+               const __nv_bfloat16 *__restrict__ gin, int ldc, float *colpart, int *err) {
   constexpr int NCOLS = N < 32 ? 32 : N;       // TMEM columns (power of two >= 32)
   constexpr uint32_t SB = N * K * 2, SA = TM * K * 2;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -132,6 +160,8 @@ gemm_tc_kernel(const __nv_bfloat16 *__restrict__ A, int lda, const __nv_bfloat16
   uint8_t *sA = smem + SB;
   uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + SB + SA);
   uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + SB + SA + 8);
+  // column sums of the CTA's rows, one row per lane group: [4][N]
+  float *sCol = reinterpret_cast<float *>(smem + SB + SA + 16);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t ntiles = (M + TM - 1) / TM;
 
@@ -144,6 +174,7 @@ gemm_tc_kernel(const __nv_bfloat16 *__restrict__ A, int lda, const __nv_bfloat16
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(su32(mbar)));
     asm volatile("fence.mbarrier_init.release.cluster;\n");
   }
+  for (int i = threadIdx.x; i < 4 * N; i += kTcThreads) sCol[i] = 0.f;
   load_tile<K>(sB, B, ldb, N, N);
   asm volatile("cp.async.commit_group;\n");
   asm volatile("tcgen05.fence::before_thread_sync;\n");
@@ -201,11 +232,14 @@ gemm_tc_kernel(const __nv_bfloat16 *__restrict__ A, int lda, const __nv_bfloat16
     if (failed) break;
     if (tile + gridDim.x < ntiles) copy_a(tile + gridDim.x);
     asm volatile("tcgen05.fence::after_thread_sync;\n");
-    const int64_t row = m0 + warp * 32 + lane;
+    // a warp reaches the 32 accumulator rows of its lane group (warp % 4); the
+    // warps of a group take 16-column pieces in turn
+    const int lg = warp & 3;
+    const int64_t row = m0 + lg * 32 + lane;
 #pragma unroll 1
-    for (int c0 = 0; c0 < N; c0 += 16) {
+    for (int c0 = (warp >> 2) * 16; c0 < N; c0 += 16 * kColGroups) {
       uint32_t r[16];
-      const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
+      const uint32_t taddr = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)c0;
       asm volatile(
           "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
           "%14,%15}, [%16];\n"
@@ -214,13 +248,13 @@ gemm_tc_kernel(const __nv_bfloat16 *__restrict__ A, int lda, const __nv_bfloat16
             "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
           : "r"(taddr));
       asm volatile("tcgen05.wait::ld.sync.aligned;\n");
+      float v[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] = row < M ? __uint_as_float(r[j]) : 0.f;
       if (row < M) {
         // 16 consecutive columns of this thread's row: 16-byte vector loads
         // of the bias and 16-byte stores (32 B of BF16 or 64 B of FP32)
         const size_t o = (size_t)row * ldc + c0;
-        float v[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
         if (bias) {
 #pragma unroll
           for (int j = 0; j < 16; j += 4) {
@@ -251,11 +285,22 @@ gemm_tc_kernel(const __nv_bfloat16 *__restrict__ A, int lda, const __nv_bfloat16
         }
         if (out_bf16) store_bf16x16(out_bf16 + o, v);
       }
+      if (colpart) {
+        const float cs = warp_column_sums16(v, lane);
+        const int c = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 +
+                      ((lane >> 1) & 1);
+        if (!(lane & 1)) sCol[lg * N + c0 + c] += cs;   // this warp's cells alone
+      }
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n");
     __syncthreads();
   }
   __syncthreads();
+  if (colpart) {
+    for (int c = threadIdx.x; c < N; c += kTcThreads)
+      colpart[(size_t)blockIdx.x * N + c] =
+          (sCol[c] + sCol[N + c]) + (sCol[2 * N + c] + sCol[3 * N + c]);
+  }
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;\n");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
@@ -266,9 +311,9 @@ gemm_tc_kernel(const __nv_bfloat16 *__restrict__ A, int lda, const __nv_bfloat16
 template <int N, int K>
 cudaError_t launch_tc(const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, int ldb, int64_t M,
                       const float *bias, int act, float *out_f32, __nv_bfloat16 *out_bf16,
-                      __nv_bfloat16 *pre_bf16, const __nv_bfloat16 *gin, int ldc, cudaStream_t st,
-                      int *err) {
-  constexpr size_t smem = (size_t)N * K * 2 + (size_t)TM * K * 2 + 16;
+                      __nv_bfloat16 *pre_bf16, const __nv_bfloat16 *gin, int ldc, float *colpart,
+                      int *nparts, cudaStream_t st, int *err) {
+  constexpr size_t smem = (size_t)N * K * 2 + (size_t)TM * K * 2 + 16 + 4 * (size_t)N * 4;
   // the attribute belongs to the current device's context: set it on every
   // launch (cheap), so a first launch on another device is configured too
   cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<N, K>,
@@ -279,61 +324,88 @@ cudaError_t launch_tc(const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, i
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t ntiles = (M + TM - 1) / TM;
   const int grid = (int)(ntiles < sms ? ntiles : sms);
-  gemm_tc_kernel<N, K><<<grid, kTcThreads, smem, st>>>(A, lda, B, ldb, M, bias, act, out_f32,
-                                                       out_bf16, pre_bf16, gin, ldc, err);
+  gemm_tc_kernel<N, K><<<grid, kTcThreads, smem, st>>>(
+      A, lda, B, ldb, M, bias, act, out_f32, out_bf16, pre_bf16, gin, ldc, colpart, err);
+  if (nparts) *nparts = grid;
   note_launches(1);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-// Forward products of the MLP on tcgen05; N and K must be 64 or 256, all row
-// strides multiples of 8 elements, bias and outputs 16-byte aligned.  *err (device) is set to 1 if a CTA gave
-// up waiting for its accumulator.
+// CTAs of a gemm_nt_tc launch at most: the rows of its column-sum partials.
+int gemm_tc_max_ctas() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
+// Products of the MLP on tcgen05; N and K must be 64 or 256, all row
+// strides multiples of 8 elements, bias and outputs 16-byte aligned.
+// colpart (may be null): column sums of the result over each CTA's rows,
+// [*nparts][N] FP32, from the values before they are rounded to BF16.  *err
+// (device) is set to 1 if a CTA gave up waiting for its accumulator.
 cudaError_t gemm_nt_tc(const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, int ldb,
                        int64_t M, int N, int K, const float *bias, int act, float *out_f32,
                        __nv_bfloat16 *out_bf16, __nv_bfloat16 *pre_bf16, int ldc, cudaStream_t st,
-                       int *err, const __nv_bfloat16 *gin) {
+                       int *err, const __nv_bfloat16 *gin, float *colpart, int *nparts) {
   if (M == 0) return cudaSuccess;
   if (lda % 8 || ldb % 8 || ldc % 8 || !err || (act == 2 && !gin)) return cudaErrorInvalidValue;
   if (((uintptr_t)bias | (uintptr_t)out_f32 | (uintptr_t)out_bf16 | (uintptr_t)pre_bf16 |
        (uintptr_t)gin) % 16)
     return cudaErrorInvalidValue;
   if (N == 256 && K == 256)
-    return launch_tc<256, 256>(A, lda, B, ldb, M, bias, act, out_f32, out_bf16, pre_bf16, gin, ldc, st, err);
+    return launch_tc<256, 256>(A, lda, B, ldb, M, bias, act, out_f32, out_bf16, pre_bf16, gin, ldc, colpart, nparts, st, err);
   if (N == 256 && K == 64)
-    return launch_tc<256, 64>(A, lda, B, ldb, M, bias, act, out_f32, out_bf16, pre_bf16, gin, ldc, st, err);
+    return launch_tc<256, 64>(A, lda, B, ldb, M, bias, act, out_f32, out_bf16, pre_bf16, gin, ldc, colpart, nparts, st, err);
   if (N == 64 && K == 256)
-    return launch_tc<64, 256>(A, lda, B, ldb, M, bias, act, out_f32, out_bf16, pre_bf16, gin, ldc, st, err);
+    return launch_tc<64, 256>(A, lda, B, ldb, M, bias, act, out_f32, out_bf16, pre_bf16, gin, ldc, colpart, nparts, st, err);
   if (N == 64 && K == 64)
-    return launch_tc<64, 64>(A, lda, B, ldb, M, bias, act, out_f32, out_bf16, pre_bf16, gin, ldc, st, err);
+    return launch_tc<64, 64>(A, lda, B, ldb, M, bias, act, out_f32, out_bf16, pre_bf16, gin, ldc, colpart, nparts, st, err);
   return cudaErrorNotSupported;
 }
 
 // ------------------------------------------------------ split-K product ---
 namespace {
 
-constexpr int KC = 64;           // K elements per pipeline chunk (128 bytes per row)
+constexpr int KC = 64;           // K elements (batch rows) per pipeline chunk
 
-// copy the K chunk [k0, k0 + KC) of rows [0, rows) of a BF16 matrix (row
-// stride ld, K valid columns) into the core-matrix layout; rows >= rows and
-// columns >= K are zero-filled
-__device__ __forceinline__ void load_chunk(uint8_t *dst, const __nv_bfloat16 *src, int64_t ld,
-                                           int rows, int R, int64_t k0, int64_t K) {
-  constexpr int CC = KC / 8;   // 16-byte chunks per row
-  for (int idx = threadIdx.x; idx < R * CC; idx += kTcThreads) {
-    const int r = idx / CC, c = idx - r * CC;
-    const uint32_t off = (uint32_t)(((r >> 3) * CC + c) * 128 + (r & 7) * 16);
-    const bool ok = r < rows && k0 + c * 8 < K;
-    const __nv_bfloat16 *s = src + (ok ? (size_t)r * ld + (size_t)(k0 + c * 8) : 0);
+// Instruction descriptor with both operands MN-major (bits 15 and 16): the
+// batch is the contraction and memory holds a batch row's columns side by
+// side, so the operands come from the row-major matrices as they are, with no
+// transposed copies.
+__host__ __device__ constexpr uint32_t instr_desc_mn(int m, int n) {
+  return instr_desc(m, n) | (1u << 15) | (1u << 16);
+}
+
+// copy batch rows [k0, k0 + KC) of columns [0, cols) of a BF16 matrix (row
+// stride ld, K valid rows) into MN-major core matrices of 8 rows (K) x 16
+// bytes (8 columns): core (row group g, column chunk c) at byte (g * CC + c) *
+// 128, so neighbouring column chunks are 128 bytes apart (the descriptor's
+// stride offset) and neighbouring row groups CC * 128 (its leading offset);
+// columns >= cols and rows >= K are zero-filled.  Eight lanes take the eight
+// rows of a core (distinct banks), four neighbouring chunks 64 bytes of a row.
+template <int CC>
+__device__ __forceinline__ void load_chunk_mn(uint8_t *dst, const __nv_bfloat16 *src, int64_t ld,
+                                              int cols, int64_t k0, int64_t K) {
+  for (int idx = threadIdx.x; idx < KC * CC; idx += kTcThreads) {
+    const int r = idx & 7, c = (idx >> 3) % CC, g = (idx >> 3) / CC;
+    const uint32_t off = (uint32_t)((g * CC + c) * 128 + r * 16);
+    const int64_t m = k0 + g * 8 + r;
+    const bool ok = m < K && c * 8 < cols;
+    const __nv_bfloat16 *s = src + (ok ? (size_t)m * ld + (size_t)c * 8 : 0);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(su32(dst + off)),
                  "l"(s), "r"(ok ? 16 : 0));
   }
 }
 
-// CTA (m-tile mt, split s): D_s = A[mt rows, K slice] . B[:, K slice]^T in
-// TMEM over chunks [c0, c1) with a two-stage copy pipeline, then the FP32
-// partial [128 x N] to part[s][mt * 128 + row][col].
+// CTA (m-tile mt, split s): D_s = A[K slice, mt columns]^T . B[K slice, :] in
+// TMEM over chunks [c0, c1) through a ring of kStages buffers (the four
+// chunks of a 64-way split of 16384 rows are all in flight at once), then
+// the FP32 partial [128 x N] to part[s][mt * 128 + row][col].
+constexpr int kStages = 4;
+
 template <int N>
 __global__ void __launch_bounds__(kTcThreads, 1)
 gemm_splitk_tc_kernel(const __nv_bfloat16 *__restrict__ A, int64_t lda, int Mrows,
@@ -342,69 +414,70 @@ gemm_splitk_tc_kernel(const __nv_bfloat16 *__restrict__ A, int64_t lda, int Mrow
   constexpr int NCOLS = N < 32 ? 32 : N;
   constexpr uint32_t SA = TM * KC * 2, SB = N * KC * 2;
   extern __shared__ __align__(1024) uint8_t smem[];
-  // stage st: A at smem + st * SA, B at smem + 2 SA + st * SB
-  auto sA = [&](int st) { return smem + st * SA; };
-  auto sB = [&](int st) { return smem + 2 * SA + st * SB; };
-  uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + 2 * SA + 2 * SB);
-  uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + 2 * SA + 2 * SB + 16);
+  // stage st: A at smem + st * (SA + SB), B behind it
+  auto sA = [&](int st) { return smem + st * (SA + SB); };
+  auto sB = [&](int st) { return smem + st * (SA + SB) + SA; };
+  uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + kStages * (SA + SB));
+  uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + kStages * (SA + SB) + kStages * 8);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int mt = blockIdx.x % mtiles, sp = blockIdx.x / mtiles;
   const int64_t nchunks = (K + KC - 1) / KC;
   const int64_t c0 = (int64_t)sp * cps;
   const int64_t c1 = c0 + cps < nchunks ? c0 + cps : nchunks;
   const int rows = Mrows - mt * TM < TM ? Mrows - mt * TM : TM;
-  const __nv_bfloat16 *Am = A + (size_t)mt * TM * lda;
+  const __nv_bfloat16 *Am = A + (size_t)mt * TM;
 
+  // one copy group per chunk, empty past the last one, so that group counts
+  // and chunks agree
+  auto copy_chunk = [&](int64_t c) {
+    if (c < c1) {
+      const int st = (int)((c - c0) % kStages);
+      load_chunk_mn<TM / 8>(sA(st), Am, lda, rows, c * KC, K);
+      load_chunk_mn<N / 8>(sB(st), B, ldb, N, c * KC, K);
+    }
+    asm volatile("cp.async.commit_group;\n");
+  };
+  for (int q = 0; q < kStages - 1; ++q) copy_chunk(c0 + q);
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                      su32(tslot)), "r"(NCOLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
   }
   if (threadIdx.x == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(su32(&mbar[0])));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(su32(&mbar[1])));
+    for (int q = 0; q < kStages; ++q)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(su32(&mbar[q])));
     asm volatile("fence.mbarrier_init.release.cluster;\n");
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n");
   const uint32_t tmem = *tslot;
-  const uint32_t idesc = instr_desc(TM, N);
-  uint32_t phase[2] = {0u, 0u};
+  const uint32_t idesc = instr_desc_mn(TM, N);
   bool failed = false;
   int last_stage = -1;
+  uint32_t last_phase = 0u;
 
-  if (c0 < c1) {
-    load_chunk(sA(0), Am, lda, rows, TM, c0 * KC, K);
-    load_chunk(sB(0), B, ldb, N, N, c0 * KC, K);
-    asm volatile("cp.async.commit_group;\n");
-  }
   for (int64_t c = c0; c < c1; ++c) {
-    const int st = (int)((c - c0) & 1);
-    if (c + 1 < c1) {
-      const int nst = st ^ 1;
-      if (c > c0) {
-        // stage nst held chunk c - 1: its products must be done before reuse
-        const bool ok = wait_parity_bounded(&mbar[nst], phase[nst]);
-        failed = __syncthreads_or(!ok) != 0;
-        if (failed) break;       // last_stage == nst: the wait below retries this phase
-        phase[nst] ^= 1u;
-      }
-      load_chunk(sA(nst), Am, lda, rows, TM, (c + 1) * KC, K);
-      load_chunk(sB(nst), B, ldb, N, N, (c + 1) * KC, K);
-      asm volatile("cp.async.commit_group;\n");
-      asm volatile("cp.async.wait_group 1;\n");
-    } else {
-      asm volatile("cp.async.wait_group 0;\n");
+    const int64_t i = c - c0;
+    const int st = (int)(i % kStages);
+    if (c > c0) {
+      // the stage of chunk c + kStages - 1 held chunk c - 1, whose products
+      // must be done (its commit: use (i - 1) / kStages of that stage)
+      const bool ok = c + kStages - 1 >= c1 || wait_parity_bounded(&mbar[last_stage], last_phase);
+      failed = __syncthreads_or(!ok) != 0;
+      if (failed) break;       // the wait below retries this phase
     }
+    copy_chunk(c + kStages - 1);
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(kStages - 1));   // chunk c has landed
     asm volatile("fence.proxy.async.shared::cta;\n");
     __syncthreads();
     if (threadIdx.x == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;\n");
 #pragma unroll
       for (int ks = 0; ks < KC / 16; ++ks) {
-        const uint64_t da = smem_desc(su32(sA(st)) + ks * 256, 128, (KC / 8) * 128);
-        const uint64_t db = smem_desc(su32(sB(st)) + ks * 256, 128, (KC / 8) * 128);
+        // two row groups of 8 per product: leading offset between them
+        const uint64_t da = smem_desc(su32(sA(st)) + ks * 2 * TM * 16, TM * 16, 128);
+        const uint64_t db = smem_desc(su32(sB(st)) + ks * 2 * N * 16, N * 16, 128);
         const uint32_t accum = (c > c0 || ks > 0) ? 1u : 0u;
         asm volatile(
             "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
@@ -416,25 +489,27 @@ gemm_splitk_tc_kernel(const __nv_bfloat16 *__restrict__ A, int64_t lda, int Mrow
               su32(&mbar[st])));
     }
     last_stage = st;
+    last_phase = (uint32_t)((i / kStages) & 1);
   }
   if (!failed && last_stage >= 0) {
     // the last commit covers every product issued before it
-    const bool ok = wait_parity_bounded(&mbar[last_stage], phase[last_stage]);
+    const bool ok = wait_parity_bounded(&mbar[last_stage], last_phase);
     failed = __syncthreads_or(!ok) != 0;
   }
   if (failed) {
     if (threadIdx.x == 0) atomicCAS(err, 0, 1);
     // give products still in flight a second bounded wait before the TMEM
     // is released, and let the copies land
-    if (last_stage >= 0) wait_parity_bounded(&mbar[last_stage], phase[last_stage]);
+    if (last_stage >= 0) wait_parity_bounded(&mbar[last_stage], last_phase);
     asm volatile("cp.async.wait_group 0;\n");
   } else if (last_stage >= 0) {
     asm volatile("tcgen05.fence::after_thread_sync;\n");
-    float *out = part + ((size_t)sp * mtiles * TM + (size_t)mt * TM + warp * 32 + lane) * N;
+    const int lg = warp & 3;
+    float *out = part + ((size_t)sp * mtiles * TM + (size_t)mt * TM + lg * 32 + lane) * N;
 #pragma unroll 1
-    for (int cc = 0; cc < N; cc += 16) {
+    for (int cc = (warp >> 2) * 16; cc < N; cc += 16 * kColGroups) {
       uint32_t r[16];
-      const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)cc;
+      const uint32_t taddr = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)cc;
       asm volatile(
           "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
           "%14,%15}, [%16];\n"
@@ -459,24 +534,42 @@ gemm_splitk_tc_kernel(const __nv_bfloat16 *__restrict__ A, int64_t lda, int Mrow
   }
 }
 
-// out[i][j] = sum over splits s (in order) of part[s][i][j], i < Mrows
-__global__ void splitk_reduce_kernel(const float *part, int splits, int mtiles, int Mrows, int N,
-                                     float *out) {
-  const int64_t total = (int64_t)Mrows * N;
-  const size_t stride = (size_t)mtiles * TM * N;
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total;
-       q += (int64_t)gridDim.x * blockDim.x) {
-    float acc = 0.f;
-    for (int s = 0; s < splits; ++s) acc += part[(size_t)s * stride + q];
-    out[q] = acc;
+// out[q] = sum over splits s of part[s][q], q < total; and, for the layer's
+// bias gradient, bout[c] = sum over p of bpart[p][c], c < nb.  A block takes
+// 64 outputs side by side; its four groups of 64 threads each sum a quarter
+// of the partials in order, and the quarters are added in order (fixed order,
+// so the result does not depend on timing).  Four quarters instead of one
+// chain: the loads of 64 to 152 partials are the time here.
+constexpr int kRedOut = 64;
+__global__ void __launch_bounds__(256) splitk_reduce_kernel(
+    const float *part, int splits, size_t stride, int total, float *out, const float *bpart,
+    int nparts, int nb, float *bout) {
+  __shared__ float sh[4][kRedOut];
+  const int lane = threadIdx.x & (kRedOut - 1), quarter = threadIdx.x / kRedOut;
+  const int wblocks = total / kRedOut;
+  const bool bias = (int)blockIdx.x >= wblocks;
+  const float *src = bias ? bpart : part;
+  const int q = (bias ? (int)blockIdx.x - wblocks : (int)blockIdx.x) * kRedOut + lane;
+  const int n = bias ? nparts : splits;
+  const size_t step = bias ? (size_t)nb : stride;
+  const int per = (n + 3) / 4, s1 = min(n, (quarter + 1) * per);
+  float acc = 0.f;
+#pragma unroll 16
+  for (int s = quarter * per; s < s1; ++s) acc += src[(size_t)s * step + q];
+  sh[quarter][lane] = acc;
+  __syncthreads();
+  if (quarter == 0) {
+    const float v = (sh[0][lane] + sh[1][lane]) + (sh[2][lane] + sh[3][lane]);
+    if (bias) bout[q] = v;
+    else out[q] = v;
   }
 }
 
 template <int N>
 cudaError_t launch_splitk(const __nv_bfloat16 *A, int64_t lda, int Mrows, const __nv_bfloat16 *B,
                           int64_t ldb, int64_t K, float *out, float *scratch, size_t scratch_bytes,
-                          cudaStream_t st, int *err) {
-  constexpr size_t smem = 2 * (size_t)TM * KC * 2 + 2 * (size_t)N * KC * 2 + 32;
+                          const float *bpart, int nparts, float *bout, cudaStream_t st, int *err) {
+  constexpr size_t smem = kStages * ((size_t)TM * KC * 2 + (size_t)N * KC * 2 + 8) + 16;
   cudaError_t e = cudaFuncSetAttribute(gemm_splitk_tc_kernel<N>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -493,29 +586,35 @@ cudaError_t launch_splitk(const __nv_bfloat16 *A, int64_t lda, int Mrows, const 
   const int splits = (int)((nchunks + cps - 1) / cps);
   gemm_splitk_tc_kernel<N><<<splits * mtiles, kTcThreads, smem, st>>>(A, lda, Mrows, B, ldb, K,
                                                                        cps, mtiles, scratch, err);
-  const int64_t total = (int64_t)Mrows * N;
-  const int rg = (int)std::min<int64_t>((total + 255) / 256, (int64_t)sms * 8);
-  splitk_reduce_kernel<<<rg, 256, 0, st>>>(scratch, splits, mtiles, Mrows, N, out);
+  // Mrows and N are 64 or 256: whole blocks of kRedOut outputs
+  splitk_reduce_kernel<<<(Mrows * N + Mrows) / kRedOut, 256, 0, st>>>(
+      scratch, splits, (size_t)mtiles * TM * N, Mrows * N, out, bpart, nparts, Mrows, bout);
   note_launches(2);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-// Weight-gradient product on tcgen05: out[Mrows x N] (FP32, row-major) =
-// A[Mrows x K] . B[N x K]^T, both BF16 K-contiguous (row strides lda, ldb,
-// multiples of 8), K any multiple of 8 (the batch), N 64 or 256, Mrows at
-// most 256.  The K range is split over CTAs; each writes an FP32 partial to
-// `scratch` and a fixed-order sum reduces them (deterministic).  *err
+// Weight and bias gradient of a layer on tcgen05: out[Mrows x N] (FP32,
+// row-major) = A^T B with A [K x Mrows] and B [K x N] BF16 row-major (row
+// strides lda, ldb, multiples of 8), K (the batch) any number of rows, N 64
+// or 256, Mrows 64 or 256; bout[Mrows] = the sum of the nparts rows of bpart
+// (column-sum partials of A's FP32 values).  The K range is split over CTAs;
+// each writes an FP32 partial to `scratch` and a fixed-order sum reduces them
+// (deterministic).  The operands are read MN-major, so the batch needs no
+// transposed copies (16384 rows: ten transposes were 100 us of a pass).  *err
 // (device) is set to 1 if a CTA gave up waiting for its products.
 cudaError_t gemm_tn_splitk_tc(const __nv_bfloat16 *A, int64_t lda, int Mrows,
                               const __nv_bfloat16 *B, int64_t ldb, int N, int64_t K, float *out,
-                              float *scratch, size_t scratch_bytes, cudaStream_t st, int *err) {
+                              float *scratch, size_t scratch_bytes, const float *bpart, int nparts,
+                              float *bout, cudaStream_t st, int *err) {
   if (K == 0 || Mrows == 0) return cudaSuccess;
-  if (lda % 8 || ldb % 8 || K % 8 || !err || Mrows > 256 || ((uintptr_t)scratch % 16))
+  if (lda % 8 || ldb % 8 || !err || (Mrows != 64 && Mrows != 256) || ((uintptr_t)scratch % 16) ||
+      !bpart || !bout)
     return cudaErrorInvalidValue;
-  if (N == 256) return launch_splitk<256>(A, lda, Mrows, B, ldb, K, out, scratch, scratch_bytes, st, err);
-  if (N == 64) return launch_splitk<64>(A, lda, Mrows, B, ldb, K, out, scratch, scratch_bytes, st, err);
+  if (((uintptr_t)A | (uintptr_t)B) % 16) return cudaErrorInvalidValue;
+  if (N == 256) return launch_splitk<256>(A, lda, Mrows, B, ldb, K, out, scratch, scratch_bytes, bpart, nparts, bout, st, err);
+  if (N == 64) return launch_splitk<64>(A, lda, Mrows, B, ldb, K, out, scratch, scratch_bytes, bpart, nparts, bout, st, err);
   return cudaErrorNotSupported;
 }
 

@@ -190,3 +190,36 @@ def test_fused_tcgen05_forward_equals_layer_by_layer(gpu, M):
     net.set_engine(2)
     np.testing.assert_array_equal(y2, net.forward(x).cpu().numpy())
     assert not np.array_equal(y2, y_fused)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", [(37, 256, 4, 3), (5, 64, 2, 64), (300, 256, 2, 5), (37, 128, 1, 2)])
+@pytest.mark.parametrize("M", [32, 96, 128, 288, 16_448])
+def test_gradients_at_the_edges_of_chunks_and_routes(gpu, M, shape):
+    """Batches below, at and past a 64-row chunk, a 128-row tile and one
+    chunk per split (16448 rows: more than 64 splits of four chunks); layer
+    shapes all on tcgen05, all on mma.sync, and changing between the two from
+    one layer to the next.  Tolerance of the comparison above."""
+    pg, torch = gpu
+    n_in, width, depth, n_out = shape
+    o = MLPOracle(n_in, width, depth, n_out)
+    rng = np.random.default_rng(M + n_in)
+    p = _random_params(o, rng).astype(np.float32)
+    pw = p.copy()
+    for wo, bo in o.offsets:
+        pw[wo:bo] = bf16_round(pw[wo:bo])
+    x = rng.normal(size=(M, n_in)).astype(np.float32)
+    t = rng.normal(size=(M, n_out)).astype(np.float32)
+    oloss, og = o.grad(pw, bf16_round(x).astype(np.float64), t.astype(np.float64))
+    xd, td = torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda()
+    for engine in (0, 1):
+        net = pg.MLP(n_in, width, depth, n_out, seed=7)
+        net.set_engine(engine)
+        net.set_params(p)
+        loss, g = net.grad(xd, td)
+        assert abs(loss - oloss) <= 3e-2 * abs(oloss)
+        for l, (wo, bo) in enumerate(o.offsets):
+            _close(g[wo:bo], og[wo:bo])
+            _close(g[bo:bo + o.dout[l]], og[bo:bo + o.dout[l]])
+        again = net.grad(xd, td)[1]
+        np.testing.assert_array_equal(again, g)      # fixed-order sums
