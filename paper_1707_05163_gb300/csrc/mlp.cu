@@ -434,7 +434,7 @@ cudaError_t mlp_fused_pack(const __nv_bfloat16 *const w[5], uint8_t *out, cudaSt
 cudaError_t mlp_fused_forward(const float *x, int64_t M, int n_in, const uint8_t *wpk,
                               const float *const bias[5], float *y, int n_out, cudaStream_t st,
                               int *err);
-cudaError_t mlp_fused_step_launch(const SurrogateStepIO &io, const uint8_t *wpk,
+cudaError_t mlp_fused_step_launch(const SurrogateStepIO &io, uint8_t *xpk, const uint8_t *wpk,
                                   const float *const bias[5], cudaStream_t st, int *err);
 cudaError_t mlp_wait_probe(long long polls, int *err, cudaStream_t st);
 cudaError_t gemm_tn_splitk_tc(const __nv_bfloat16 *A, int64_t lda, int Mrows,
@@ -641,13 +641,13 @@ static cudaError_t ensure_packed(pg_mlp *n, cudaStream_t st) {
 
 bool mlp_fused_step_ok(const pg_mlp *n) { return n && fused_shape(n) && n->n_in == 37 && n->n_out == 3; }
 
-pg_status mlp_fused_step(pg_mlp *n, const SurrogateStepIO &io, cudaStream_t st) {
+pg_status mlp_fused_step(pg_mlp *n, const SurrogateStepIO &io, uint8_t *xpk, cudaStream_t st) {
   if (!mlp_fused_step_ok(n)) { set_error("network cannot run the fused step"); return PG_ERR_ARG; }
   CUM(ensure_packed(n, st));
   const float *bias[5];
   for (int l = 0; l < 5; ++l) bias[l] = n->w + n->boff[l];
   CUM(cudaMemsetAsync(io.ferr, 0, 4, st));
-  CUM(mlp_fused_step_launch(io, n->wpk, bias, st, n->d_err));
+  CUM(mlp_fused_step_launch(io, xpk, n->wpk, bias, st, n->d_err));
   int err[2] = {0, 0};
   CUM(cudaMemcpyAsync(&err[0], n->d_err, 4, cudaMemcpyDeviceToHost, st));
   CUM(cudaMemcpyAsync(&err[1], io.ferr, 4, cudaMemcpyDeviceToHost, st));

@@ -301,8 +301,13 @@ pg_status pg_surrogate_run(pg_pset *ps, pg_mlp *net, const pg_kernel *k, int nst
   const int64_t n = ps->n;
   const int sm = ps->fs->sm_count;
   pg_surrogate_stats S{};
-  // buffers: features, outputs, reject flags, checkpoint and check sets
+  // a network step: features, network, displacement -- two launches for the
+  // surrogate's network shape on tcgen05, else three kernels
+  const bool fused_step = mlp_fused_step_ok(net);
+  // buffers: features (packed, or with the outputs), reject flags, checkpoint
+  // and check sets
   float *x = nullptr, *y = nullptr;
+  uint8_t *xpk = nullptr;
   uint8_t *rej = nullptr;
   double *esum = nullptr;
   unsigned long long *nrej = nullptr;
@@ -313,15 +318,20 @@ pg_status pg_surrogate_run(pg_pset *ps, pg_mlp *net, const pg_kernel *k, int nst
   CUS(cudaEventCreate(&e1));
   CUS(cudaEventCreate(&e2));
   auto cleanup = [&]() {
-    dev_free(x); dev_free(y); dev_free(rej); dev_free(esum); dev_free(nrej);
+    dev_free(x); dev_free(y); dev_free(xpk); dev_free(rej); dev_free(esum); dev_free(nrej);
     dev_free(flags); dev_free(offs); dev_free(scan_tmp); dev_free(idx);
     if (ckpt) pg_pset_destroy(ckpt);
     if (chk) pg_pset_destroy(chk);
     if (rset) pg_pset_destroy(rset);
     cudaEventDestroy(e0); cudaEventDestroy(e1); cudaEventDestroy(e2);
   };
-  cudaError_t e = dev_alloc((void **)&x, (size_t)std::max<int64_t>(n, 1) * kFeat * 4);
-  if (e == cudaSuccess) e = dev_alloc((void **)&y, (size_t)std::max<int64_t>(n, 1) * 3 * 4);
+  cudaError_t e = cudaSuccess;
+  if (fused_step) {
+    e = dev_alloc((void **)&xpk, mlp_fused_step_scratch(n));
+  } else {
+    e = dev_alloc((void **)&x, (size_t)std::max<int64_t>(n, 1) * kFeat * 4);
+    if (e == cudaSuccess) e = dev_alloc((void **)&y, (size_t)std::max<int64_t>(n, 1) * 3 * 4);
+  }
   if (e == cudaSuccess) e = dev_alloc((void **)&rej, (size_t)std::max<int64_t>(n, 1));
   if (e == cudaSuccess) e = dev_alloc((void **)&esum, 16);
   if (e == cudaSuccess) e = dev_alloc((void **)&nrej, 8);
@@ -369,9 +379,6 @@ pg_status pg_surrogate_run(pg_pset *ps, pg_mlp *net, const pg_kernel *k, int nst
     dst->t_max = src->t_max;
     return q;
   };
-  // a network step: features, network, displacement -- one fused tcgen05
-  // kernel for the surrogate's network shape, else three kernels
-  const bool fused_step = mlp_fused_step_ok(net);
   auto network_step = [&]() -> pg_status {
     if (fused_step) {
       SurrogateStepIO io;
@@ -380,7 +387,7 @@ pg_status pg_surrogate_run(pg_pset *ps, pg_mlp *net, const pg_kernel *k, int nst
       io.lon = (float *)ps->x; io.lat = (float *)ps->y; io.dep = (float *)ps->z;
       io.time = ps->time; io.step = ps->step; io.status = ps->status;
       io.n = ps->n; io.horizon = horizon; io.ferr = ps->d_err;
-      const pg_status q = mlp_fused_step(net, io, st);
+      const pg_status q = mlp_fused_step(net, io, xpk, st);
       if (!q) { ps->t_min += horizon; ps->t_max += horizon; }
       return q;
     }

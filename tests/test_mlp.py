@@ -223,3 +223,24 @@ def test_gradients_at_the_edges_of_chunks_and_routes(gpu, M, shape):
             _close(g[bo:bo + o.dout[l]], og[bo:bo + o.dout[l]])
         again = net.grad(xd, td)[1]
         np.testing.assert_array_equal(again, g)      # fixed-order sums
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("tiles,extra", [(1, 0), (1, 1), (2, -127), (2, 0), (2, 1), (3, 0)])
+def test_fused_forward_with_lone_and_paired_tiles(gpu, tiles, extra):
+    """One, two and three 128-row tiles per multiprocessor, and one tile more
+    or a ragged last one: CTAs with a pair of tiles, a tile alone, a pair and
+    a tile alone.  Bit for bit the layer-by-layer forward; 64, 1 and 16
+    inputs and outputs at the limits of the kernel's shape."""
+    pg, torch = gpu
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    M = tiles * sms * 128 + extra
+    for n_in, n_out in ((37, 3), (64, 16), (1, 1)):
+        net = pg.MLP(n_in, 256, 4, n_out, seed=17)
+        x = torch.randn(M, n_in, device="cuda", generator=torch.Generator("cuda").manual_seed(M))
+        net.set_engine(2)
+        want = net.forward(x)
+        net.set_engine(1)
+        got = net.forward(x)
+        assert torch.equal(got, want)
+        assert torch.equal(net.forward(x), got)
