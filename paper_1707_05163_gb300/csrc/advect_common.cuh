@@ -91,6 +91,33 @@ __device__ __forceinline__ float cos_deg(float lat) {
   return fmaf(x2, p, 1.0f);
 }
 
+// FP64 a / d, correctly rounded, for a divisor used many times, from r =
+// RN(1 / d): Markstein's correction (P. W. Markstein, IBM J. Res. Dev. 34(1),
+// 1990) -- q = a r, corrected once by its remainder, is within one unit in the
+// last place, and the second correction then rounds as the division does
+// (five instructions of the FP64 pipe, without a branch).  Dividends outside
+// 2^-639 .. 2^641 (zero, infinite and NaN ones among them) and divisors
+// whose reciprocal is marked unfit (0) are divided.
+__device__ __forceinline__ double reciprocal_for(double d) {
+  const unsigned e = ((unsigned)__double2hiint(d) >> 20) & 0x7ffu;
+  return e - 0x2ffu <= 0x200u ? 1.0 / d : 0.0;         // 2^-256 .. 2^257
+}
+__device__ __forceinline__ double quotient_refined(double a, double d, double r) {
+  double q = a * r;
+  q = fma(fma(-d, q, a), r, q);
+  return fma(fma(-d, q, a), r, q);
+}
+__device__ __forceinline__ bool dividend_fit(double a) {
+  return (((unsigned)__double2hiint(a) >> 20) & 0x7ffu) - 0x180u <= 0x500u;
+}
+__device__ __forceinline__ double quotient(double a, double d, double r) {
+  if (!dividend_fit(a) | (__double2hiint(r) == 0)) return a / d;
+  return quotient_refined(a, d, r);
+}
+__device__ __forceinline__ double quotient6(double a) {
+  return dividend_fit(a) ? quotient_refined(a, 6.0, 1.0 / 6.0) : a / 6.0;
+}
+
 // u (m/s) -> degrees/s of longitude at latitude lat; v (m/s) -> degrees/s.
 __device__ __forceinline__ double lon_rate(double u, double lat, const KernArgs &k) {
   return u / (k.deg_m * cos_deg(lat));
@@ -98,7 +125,9 @@ __device__ __forceinline__ double lon_rate(double u, double lat, const KernArgs 
 __device__ __forceinline__ float lon_rate(float u, float lat, const KernArgs &k) {
   return __fdividef(u, k.deg_m_f * cos_deg(lat));
 }
-__device__ __forceinline__ double lat_rate(double v, const KernArgs &k) { return v / k.deg_m; }
+__device__ __forceinline__ double lat_rate(double v, const KernArgs &k) {
+  return dividend_fit(v) ? quotient_refined(v, k.deg_m, k.inv_deg_m) : v / k.deg_m;
+}
 __device__ __forceinline__ float lat_rate(float v, const KernArgs &k) { return v * k.inv_deg_m_f; }
 
 template <typename Real> __device__ __forceinline__ const Real *axis(const GridArgs &g, int a);
@@ -151,7 +180,8 @@ struct Sampler {
   // cached cell (ci = -1: none) and its bounds
   int ci, cj, ck;
   Real xlo, xhi, ylo, yhi, zlo, zhi;
-  Real rx, ry, rz;            // 1 / (hi - lo), FP32 path only
+  Real rx, ry, rz;            // 1 / (hi - lo)
+  Real dx, dy, dz;            // hi - lo, FP64 path only
   // cached snapshot interval and the snapshots whose corners are held
   int s0;                     // first snapshot of the cached pair (second: snap_next)
   // what `v` lacks: 1 the cell changed, 2 the snapshot pair moved on by one
@@ -174,9 +204,12 @@ struct Sampler {
 // FP32: stage positions are at most one turn away, so a compare and one
 // add/subtract do (fmod for anything farther).
 __device__ __forceinline__ double wrap_lon(double p, double x0) {
-  double r = fmod(p - x0, 360.0);
-  if (r < 0.0) r += 360.0;
-  if (r >= 360.0) r -= 360.0;
+  double r = p - x0;
+  if (!(r >= 0.0 && r < 360.0)) {       // fmod is the identity on [0, 360)
+    r = fmod(r, 360.0);
+    if (r < 0.0) r += 360.0;
+    if (r >= 360.0) r -= 360.0;
+  }
   return x0 + r;
 }
 __device__ __forceinline__ float wrap_lon(float p, float x0) {

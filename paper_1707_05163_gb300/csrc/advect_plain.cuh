@@ -26,8 +26,11 @@
 
 namespace pg {
 
-// Locate p on the longitude axis, using and refreshing the cache.
-// Returns false when the position is out of the domain.
+// FP64: locate p on the longitude axis, using and refreshing the cache.
+// Returns false when the position is out of the domain.  The cached cell is
+// tested first: a position inside it is inside the domain.  (The FP64 pipe
+// takes a warp instruction every 16 clocks of an SM, comparisons included, so
+// the stage's time is its count of FP64 instructions.)
 template <typename Real, typename Store, int NF, bool D3, int GEO>
 __device__ __forceinline__ bool locate_lon(const GridArgs &g, Sampler<Real, Store, NF, D3, GEO> &c,
                                            Real p, Real &xi) {
@@ -36,10 +39,9 @@ __device__ __forceinline__ bool locate_lon(const GridArgs &g, Sampler<Real, Stor
   if (is_per<GEO>(g)) {
     if (!isfinite(p)) return false;
     q = wrap_lon(p, axis_lo(g, 0, p));
-  } else if (!(p >= axis_lo(g, 0, p) && p <= axis_hi(g, 0, p))) {
-    return false;
   }
   if (!(c.ci >= 0 && in_cell<Real>(q, c.xlo, c.xhi, c.ci == g.nx - 2 && !is_per<GEO>(g)))) {
+    if (!is_per<GEO>(g) && !(p >= axis_lo(g, 0, p) && p <= axis_hi(g, 0, p))) return false;
     c.dirty |= 1;
     if (is_per<GEO>(g) && q >= axis_hi(g, 0, p)) {
       c.ci = g.nx - 1;
@@ -50,26 +52,27 @@ __device__ __forceinline__ bool locate_lon(const GridArgs &g, Sampler<Real, Stor
       c.ci = i;
       c.xlo = x[i]; c.xhi = x[i + 1];
     }
-    c.rx = (Real)1 / (c.xhi - c.xlo);
+    c.dx = c.xhi - c.xlo;
+    c.rx = reciprocal_for(c.dx);
   }
-  if constexpr (sizeof(Real) == 8) xi = (q - c.xlo) / (c.xhi - c.xlo);
-  else xi = (q - c.xlo) * c.rx;
+  xi = quotient(q - c.xlo, c.dx, c.rx);
   return true;
 }
 
 template <typename Real>
 __device__ __forceinline__ bool locate_axis(const GridArgs &g, int a, int n, int &ci, Real &lo,
-                                            Real &hi, Real &rinv, Real p, Real &xi, int &dirty) {
+                                            Real &hi, Real &d, Real &rinv, Real p, Real &xi,
+                                            int &dirty) {
   const Real *x = axis<Real>(g, a);
   if (!(ci >= 0 && in_cell<Real>(p, lo, hi, ci == n - 2))) {
     if (!(p >= x[0] && p <= x[n - 1])) return false;
     const int i = axis_search<Real>(g, a, n, p);
     ci = i; lo = x[i]; hi = x[i + 1];
     dirty |= 1;
-    rinv = (Real)1 / (hi - lo);
+    d = hi - lo;
+    rinv = reciprocal_for(d);
   }
-  if constexpr (sizeof(Real) == 8) xi = (p - lo) / (hi - lo);
-  else xi = (p - lo) * rinv;
+  xi = quotient(p - lo, d, rinv);
   return true;
 }
 
@@ -226,9 +229,9 @@ __device__ __forceinline__ int velocity(const A &a, Sampler<Real, Store, NF, D3,
   }
   Real xi, eta, zeta = (Real)0;
   if (!locate_lon(g, c, lon, xi)) return 1;
-  if (!locate_axis<Real>(g, 1, g.ny, c.cj, c.ylo, c.yhi, c.ry, lat, eta, c.dirty)) return 1;
+  if (!locate_axis<Real>(g, 1, g.ny, c.cj, c.ylo, c.yhi, c.dy, c.ry, lat, eta, c.dirty)) return 1;
   if constexpr (D3) {
-    if (!locate_axis<Real>(g, 2, g.nz, c.ck, c.zlo, c.zhi, c.rz, dep, zeta, c.dirty)) return 2;
+    if (!locate_axis<Real>(g, 2, g.nz, c.ck, c.zlo, c.zhi, c.dz, c.rz, dep, zeta, c.dirty)) return 2;
   } else {
     c.ck = 0;
   }
@@ -292,7 +295,7 @@ __device__ __forceinline__ int step_one(const A &a, Sampler<Real, Store, NF, D3,
     if (s > 0) {
       px = lon + kc[0] * off;
       py = lat + kc[1] * off;
-      pz = dep + kc[2] * off;
+      if constexpr (NF == 3) pz = dep + kc[2] * off;
     }
     if ((r = velocity<EXT>(a, c, ck, off, px, py, pz, kc))) return r;
     if (s == 0) {
@@ -300,9 +303,10 @@ __device__ __forceinline__ int step_one(const A &a, Sampler<Real, Store, NF, D3,
     } else if (s == 3) {
       acc[0] = acc[0] + kc[0]; acc[1] = acc[1] + kc[1]; acc[2] = acc[2] + kc[2];
     } else {
-      acc[0] = acc[0] + (Real)2 * kc[0];
-      acc[1] = acc[1] + (Real)2 * kc[1];
-      acc[2] = acc[2] + (Real)2 * kc[2];
+      // 2 k is exact, so one rounding either way
+      acc[0] = fma((Real)2, kc[0], acc[0]);
+      acc[1] = fma((Real)2, kc[1], acc[1]);
+      acc[2] = fma((Real)2, kc[2], acc[2]);
     }
   }
   Real nlon, nlat, ndep;
@@ -317,9 +321,10 @@ __device__ __forceinline__ int step_one(const A &a, Sampler<Real, Store, NF, D3,
     nlat = lat + acc[1] * hr;
     ndep = dep + acc[2] * hr;
   } else {
-    nlon = lon + acc[0] / (Real)6 * hr;
-    nlat = lat + acc[1] / (Real)6 * hr;
-    ndep = dep + acc[2] / (Real)6 * hr;
+    nlon = lon + quotient6(acc[0]) * hr;
+    nlat = lat + quotient6(acc[1]) * hr;
+    // two fields have no vertical velocity: acc[2] / 6 h is a zero
+    ndep = dep + (NF == 3 ? quotient6(acc[2]) : (Real)0) * hr;
   }
   return finish_step<EXT, Real, Store, NF, D3, GEO>(a, lon, lat, dep, nlon, nlat, ndep, hr, h64,
                                                     age, idp, stp);
@@ -563,9 +568,12 @@ __device__ __forceinline__ unsigned long long advance_particle(const A &a, int64
       }
     } else if constexpr (sizeof(Real) == 8) {
       // FP64: the definition's loop, time accumulated step by step.
-      while (sgn * (a.t_stop - t) > 0.0 && sgn * (a.t_end - t) > 0.0) {
+      const bool fwd = a.dt > 0.0;
+      const double lim = fwd ? fmin(a.t_stop, a.t_end) : fmax(a.t_stop, a.t_end);
+      while (fwd ? t < lim : t > lim) {
         double h = a.dt;
-        if (sgn * (a.t_end - t) < sgn * h) h = a.t_end - t;
+        const double left = a.t_end - t;
+        if (fwd ? left < h : left > h) h = left;
         ck.t = t;
         const int r = step_one<EXT>(a, c, ck, lon, lat, dep, (Real)h, h, age, idp, stp);
         if (r == STATUS_DELETED) {      // taken, then deleted by the age behaviour

@@ -388,3 +388,26 @@ def test_error_conventions(pg):
     with pytest.raises(pg.PGError) as e:
         ps2.execute(pg.Kernel("rk4"), 2.5 * DAY, 1800.0)
     assert e.value.code == -5
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 4800, 19457])
+@pytest.mark.parametrize("scale", [1.0, 3e7, 1e-90, 1e-250])
+def test_fp64_cells_of_any_width_are_bit_identical(pg, scale, n):
+    """FP64 on stretched flat axes, 3-D and time-varying, at widths whose
+    reciprocal serves for the in-cell fractions and at widths and velocities
+    so small that they are divided; particle counts around the launch's block
+    sizes.  Bit for bit the oracle."""
+    rng = np.random.default_rng(n)
+    ax = [np.cumsum(rng.uniform(0.3, 3.0, m)) * scale for m in (17, 13, 9)]
+    times = np.cumsum(rng.uniform(2e4, 5e4, 5))
+    data = rng.normal(size=(5, 3, 9, 13, 17)) * scale * 1e-6
+    spec = synth.FieldSpec(ax[0], ax[1], ax[2], times, data, 0, False, 0.0, 3, None)
+    pos = [rng.uniform(a[0], a[-1], n) for a in ax]
+    pos[0][0] = ax[0][3]                     # on a node: a fraction of zero
+    T = times[-1] - times[0]
+    o = oracle_run(oracle_field(spec), *pos, times[0], 3600.0, T)
+    fs = pg.FieldSet.from_spec(spec, storage="f64")
+    g = gpu_run(pg.ParticleSet(fs, *pos, t0=times[0], pos="f64"), pg.Kernel("rk4"), T, 3600.0)
+    assert g["steps"] == o["steps"]
+    for k in ("lon", "lat", "depth", "status", "time"):
+        np.testing.assert_array_equal(g["final"][k], o["final"][k], err_msg=k)
