@@ -15,6 +15,8 @@
 #include <cmath>
 #include <limits>
 
+#include <math_constants.h>
+
 #include "pg_host.h"
 
 namespace pg {
@@ -115,16 +117,6 @@ __global__ void f32_to_f64_kernel(const float *src, double *dst, int64_t n) {
        i += (int64_t)gridDim.x * blockDim.x)
     dst[i] = (double)src[i];
 }
-__global__ void fill_f64_kernel(double *dst, double v, int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    dst[i] = v;
-}
-__global__ void iota_u64_kernel(uint64_t *dst, uint64_t base, int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    dst[i] = base + (uint64_t)i;
-}
 
 int grid_for(int64_t n, int sm) {
   int64_t g = (n + 255) / 256;
@@ -133,50 +125,53 @@ int grid_for(int64_t n, int sm) {
   return (int)(g < 1 ? 1 : g);
 }
 
-// Copy n doubles (host or device) into a device array of the position type.
-pg_status upload_coord(const double *src, int64_t n, void *dst, int pos, double fill, int sm,
-                       cudaStream_t st) {
-  if (n == 0) return PG_OK;
-  if (pos == PG_POS_F64) {
-    if (src) {
-      CU(cudaMemcpyAsync(dst, src, n * 8, cudaMemcpyDefault, st));
-    } else {
-      fill_f64_kernel<<<grid_for(n, sm), 256, 0, st>>>((double *)dst, fill, n);
-      note_launches(1);
-      CU(cudaGetLastError());
-    }
-    return PG_OK;
+// Whether a kernel on `device` may read or write doubles at p: device or
+// managed memory of that device, aligned.
+bool kernel_ptr(const void *p, int device) {
+  if ((uintptr_t)p % 8) return false;
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
   }
-  if (!src) {
-    std::vector<float> h((size_t)n, (float)fill);
-    CU(cudaMemcpyAsync(dst, h.data(), n * 4, cudaMemcpyHostToDevice, st));
-    CU(cudaStreamSynchronize(st));
-    return PG_OK;
-  }
-  if (!is_device_ptr(src)) {
-    // host source: copy the FP64 values to the device (at the copy engines'
-    // rate from pinned memory) and round them there
-    double *tmp = nullptr;
-    CU(dev_alloc((void **)&tmp, (size_t)n * 8));
-    cudaError_t e = cudaMemcpyAsync(tmp, src, n * 8, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) {
-      f64_to_f32_kernel<<<grid_for(n, sm), 256, 0, st>>>(tmp, (float *)dst, n);
-      note_launches(1);
-      e = cudaGetLastError();
+  return (at.type == cudaMemoryTypeDevice && at.device == device) || at.type == cudaMemoryTypeManaged;
+}
+
+// New particles [0, n) of the given arrays (already offset): positions from
+// FP64 sources (x, y; z may be null: zfill) unless the set is in the cell form
+// (to_cell_kernel), the start time, consecutive ids, and the zero or NaN
+// start of everything else -- one pass instead of a launch per array.
+template <typename Real>
+__global__ void init_particles_kernel(const double *sx, const double *sy, const double *sz,
+                                      double zfill, PsetArrays A, int64_t n, bool set_time,
+                                      double t0, bool set_id, uint64_t id_base, int nvar,
+                                      int64_t vstride) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    if (sx) {
+      reinterpret_cast<Real *>(A.x)[i] = (Real)sx[i];
+      reinterpret_cast<Real *>(A.y)[i] = (Real)sy[i];
+      reinterpret_cast<Real *>(A.z)[i] = (Real)(sz ? sz[i] : zfill);
     }
-    const cudaError_t e2 = cudaStreamSynchronize(st);
-    dev_free(tmp);
-    if (e == cudaSuccess) e = e2;
-    if (e != cudaSuccess) {
-      set_error("particle upload failed: %s", cudaGetErrorString(e));
-      return PG_ERR_CUDA;
-    }
-    return PG_OK;
+    if (set_time) A.time[i] = t0;
+    if (set_id) A.id[i] = id_base + (uint64_t)i;
+    A.step[i] = 0u;
+    A.status[i] = 0;
+    A.age[i] = 0.0;
+    A.hstep[i] = 0.0;
+    for (int j = 0; j < nvar; ++j) A.var[(size_t)j * vstride + i] = CUDART_NAN;
   }
-  f64_to_f32_kernel<<<grid_for(n, sm), 256, 0, st>>>(src, (float *)dst, n);
-  note_launches(1);
-  CU(cudaGetLastError());
-  return PG_OK;
+}
+
+// State of an FP32 set into FP64 destinations (any may be null).
+__global__ void export_f32_kernel(const float *x, const float *y, const float *z, double *dx,
+                                  double *dy, double *dz, int64_t n) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    if (dx) dx[i] = (double)x[i];
+    if (dy) dy[i] = (double)y[i];
+    if (dz) dz[i] = (double)z[i];
+  }
 }
 
 }  // namespace
@@ -184,31 +179,42 @@ pg_status upload_coord(const double *src, int64_t n, void *dst, int pos, double 
 namespace pg {
 pg_status alloc_arrays(PsetArrays &A, int pos, int64_t cap, int nvar) {
   const size_t n = (size_t)std::max<int64_t>(cap, 1);
-  cudaError_t e = cudaSuccess;
-  auto al = [&](void **p, size_t b) {
-    if (e == cudaSuccess) e = dev_alloc(p, b);
+  // the arrays one after another, each on a 256-byte boundary: sizes first,
+  // then addresses
+  char *base = nullptr;
+  size_t off = 0;
+  auto place = [&](void **p, size_t b) {
+    if (base) *p = base + off;
+    off += (b + 255) / 256 * 256;
   };
-  if (pos == PG_POS_CELL) {
-    al((void **)&A.ci, n * 4); al((void **)&A.cj, n * 4); al((void **)&A.ck, n * 4);
-    al((void **)&A.fx, n * 4); al((void **)&A.fy, n * 4); al((void **)&A.fz, n * 4);
-  } else {
-    const size_t el = pos_elem(pos);
-    al(&A.x, n * el); al(&A.y, n * el); al(&A.z, n * el);
-  }
-  al((void **)&A.time, n * 8);
-  al((void **)&A.id, n * 8);
-  al((void **)&A.step, n * 4);
-  al((void **)&A.status, n);
-  al((void **)&A.age, n * 8);
-  al((void **)&A.hstep, n * 8);
-  if (nvar > 0) al((void **)&A.var, n * 8 * (size_t)nvar);
+  auto layout = [&]() {
+    off = 0;
+    if (pos == PG_POS_CELL) {
+      place((void **)&A.ci, n * 4); place((void **)&A.cj, n * 4); place((void **)&A.ck, n * 4);
+      place((void **)&A.fx, n * 4); place((void **)&A.fy, n * 4); place((void **)&A.fz, n * 4);
+    } else {
+      const size_t el = pos_elem(pos);
+      place(&A.x, n * el); place(&A.y, n * el); place(&A.z, n * el);
+    }
+    place((void **)&A.time, n * 8);
+    place((void **)&A.id, n * 8);
+    place((void **)&A.step, n * 4);
+    place((void **)&A.status, n);
+    place((void **)&A.age, n * 8);
+    place((void **)&A.hstep, n * 8);
+    if (nvar > 0) place((void **)&A.var, n * 8 * (size_t)nvar);
+  };
+  layout();
+  const cudaError_t e = dev_alloc(&A.base, off);
   if (e != cudaSuccess) {
-    A.free_all();
+    A = PsetArrays();
     cudaGetLastError();
     set_error("device allocation of %lld particles failed: %s", (long long)cap,
               cudaGetErrorString(e));
     return PG_ERR_NOMEM;
   }
+  base = (char *)A.base;
+  layout();
   return PG_OK;
 }
 
@@ -275,6 +281,7 @@ GridArgs pg::grid_args_of(const pg_fieldset *fs) { return grid_args(fs); }
 
 PsetArrays pg::pset_arrays(const pg_pset *ps) {
   PsetArrays A;
+  A.base = ps->base;
   A.x = ps->x; A.y = ps->y; A.z = ps->z;
   A.ci = ps->ci; A.cj = ps->cj; A.ck = ps->ck;
   A.fx = ps->fx; A.fy = ps->fy; A.fz = ps->fz;
@@ -284,6 +291,7 @@ PsetArrays pg::pset_arrays(const pg_pset *ps) {
 }
 
 void pg::pset_set_arrays(pg_pset *ps, const PsetArrays &A) {
+  ps->base = A.base;
   ps->x = A.x; ps->y = A.y; ps->z = A.z;
   ps->ci = A.ci; ps->cj = A.cj; ps->ck = A.ck;
   ps->fx = A.fx; ps->fy = A.fy; ps->fz = A.fz;
@@ -452,24 +460,6 @@ void free_resident(pg_fieldset *fs) {
 void free_tracers(pg_fieldset *fs) {
   for (void *p : fs->tr_slabs) dev_free(p);
   fs->tr_slabs.assign(fs->tr_slabs.size(), nullptr);
-}
-
-// Initial variables of particles [off, off + n): age 0, sampled values NaN
-// (nothing sampled yet).
-pg_status init_variables(pg_pset *ps, int64_t off, int64_t n, cudaStream_t st) {
-  if (n <= 0) return PG_OK;
-  const int sm = ps->fs->sm_count;
-  fill_f64_kernel<<<grid_for(n, sm), 256, 0, st>>>(ps->age + off, 0.0, n);
-  fill_f64_kernel<<<grid_for(n, sm), 256, 0, st>>>(ps->hstep + off, 0.0, n);
-  note_launches(2);
-  for (int j = 0; j < ps->nvar; ++j) {
-    fill_f64_kernel<<<grid_for(n, sm), 256, 0, st>>>(ps->var + (size_t)j * ps->cap + off,
-                                                     std::numeric_limits<double>::quiet_NaN(), n);
-    note_launches(1);
-  }
-  CU(cudaGetLastError());
-  CU(cudaStreamSynchronize(st));
-  return PG_OK;
 }
 
 }  // namespace
@@ -918,39 +908,60 @@ static pg_status fill_particles(pg_pset *ps, int64_t off, int64_t n, const doubl
                                 const double *lat, const double *depth, const double *time,
                                 double t0, const uint64_t *ids, uint64_t id_base,
                                 cudaStream_t st, double &tmin, double &tmax) {
-  const int sm = ps->fs->sm_count;
-  pg_status r;
-  if (ps->pos == PG_POS_CELL) {
-    // FP64 positions on the device, then split into cell index + offset
-    double *tmp = nullptr;
-    CU(dev_alloc((void **)&tmp, (size_t)n * 8 * 3));
-    r = upload_coord(lon, n, tmp, PG_POS_F64, 0.0, sm, st);
-    if (!r) r = upload_coord(lat, n, tmp + n, PG_POS_F64, 0.0, sm, st);
-    if (!r) r = upload_coord(depth, n, tmp + 2 * n, PG_POS_F64, ps->fs->depth[0], sm, st);
-    if (!r) {
-      cudaError_t e = launch_to_cell(grid_args(ps->fs), tmp, tmp + n, tmp + 2 * n, ps->ci + off,
-                                     ps->cj + off, ps->ck + off, ps->fx + off, ps->fy + off,
-                                     ps->fz + off, n, sm, st);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-      if (e != cudaSuccess) {
-        set_error("cell conversion failed: %s", cudaGetErrorString(e));
-        r = PG_ERR_CUDA;
-      }
+  const pg_fieldset *fs = ps->fs;
+  const int sm = fs->sm_count;
+  const bool cell = ps->pos == PG_POS_CELL;
+  // sources a kernel can read stay where they are; the others are copied to
+  // the device (at the copy engines' rate from pinned memory) and rounded or
+  // split there
+  const double *src[3] = {lon, lat, depth};
+  int staged = 0;
+  for (const double *p : src) staged += p && !kernel_ptr(p, fs->device);
+  double *tmp = nullptr;
+  if (staged) CU(dev_alloc((void **)&tmp, (size_t)n * 8 * staged));
+  cudaError_t e = cudaSuccess;
+  double *next = tmp;
+  for (const double *&p : src)
+    if (p && !kernel_ptr(p, fs->device)) {
+      if (e == cudaSuccess) e = cudaMemcpyAsync(next, p, n * 8, cudaMemcpyDefault, st);
+      p = next;
+      next += n;
     }
-    dev_free(tmp);
-    if (r) return r;
+  PsetArrays A = arrays_of(ps);
+  const size_t el = pos_elem(ps->pos);
+  if (cell) {
+    if (e == cudaSuccess)
+      e = launch_to_cell(grid_args(fs), src[0], src[1], src[2], ps->ci + off, ps->cj + off,
+                         ps->ck + off, ps->fx + off, ps->fy + off, ps->fz + off, n, sm, st);
+    src[0] = nullptr;
   } else {
-    const size_t el = pos_elem(ps->pos);
-    if ((r = upload_coord(lon, n, (char *)ps->x + off * el, ps->pos, 0.0, sm, st))) return r;
-    if ((r = upload_coord(lat, n, (char *)ps->y + off * el, ps->pos, 0.0, sm, st))) return r;
-    if ((r = upload_coord(depth, n, (char *)ps->z + off * el, ps->pos, 0.0, sm, st))) return r;
+    A.x = (char *)A.x + off * el; A.y = (char *)A.y + off * el; A.z = (char *)A.z + off * el;
+  }
+  A.time += off; A.id += off; A.step += off; A.status += off; A.age += off; A.hstep += off;
+  if (A.var) A.var += off;
+  if (e == cudaSuccess) {
+    auto kern = ps->pos == PG_POS_F64 ? init_particles_kernel<double> : init_particles_kernel<float>;
+    kern<<<grid_for(n, sm), 256, 0, st>>>(src[0], src[1], src[2], 0.0, A, n, time == nullptr, t0,
+                                          ids == nullptr, id_base, ps->nvar, ps->cap);
+    note_launches(1);
+    e = cudaGetLastError();
   }
   tmin = t0; tmax = t0;
+  std::vector<double> h;
+  if (e == cudaSuccess && time) {
+    h.resize((size_t)n);
+    e = cudaMemcpyAsync(ps->time + off, time, n * 8, cudaMemcpyDefault, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), time, n * 8, cudaMemcpyDefault, st);
+  }
+  if (e == cudaSuccess && ids) e = cudaMemcpyAsync(ps->id + off, ids, n * 8, cudaMemcpyDefault, st);
+  const cudaError_t e2 = cudaStreamSynchronize(st);
+  dev_free(tmp);
+  if (e == cudaSuccess) e = e2;
+  if (e != cudaSuccess) {
+    set_error("particle upload failed: %s", cudaGetErrorString(e));
+    return PG_ERR_CUDA;
+  }
   if (time) {
-    CU(cudaMemcpyAsync(ps->time + off, time, n * 8, cudaMemcpyDefault, st));
-    std::vector<double> h((size_t)n);
-    CU(cudaMemcpyAsync(h.data(), time, n * 8, cudaMemcpyDefault, st));
-    CU(cudaStreamSynchronize(st));
     tmin = std::numeric_limits<double>::infinity();
     tmax = -tmin;
     for (double v : h) {
@@ -961,21 +972,7 @@ static pg_status fill_particles(pg_pset *ps, int64_t off, int64_t n, const doubl
       tmin = std::min(tmin, v);
       tmax = std::max(tmax, v);
     }
-  } else {
-    fill_f64_kernel<<<grid_for(n, sm), 256, 0, st>>>(ps->time + off, t0, n);
-    note_launches(1);
-    CU(cudaGetLastError());
   }
-  if (ids) {
-    CU(cudaMemcpyAsync(ps->id + off, ids, n * 8, cudaMemcpyDefault, st));
-  } else {
-    iota_u64_kernel<<<grid_for(n, sm), 256, 0, st>>>(ps->id + off, id_base, n);
-    note_launches(1);
-    CU(cudaGetLastError());
-  }
-  CU(cudaMemsetAsync(ps->step + off, 0, n * 4, st));
-  CU(cudaMemsetAsync(ps->status + off, 0, n, st));
-  CU(cudaStreamSynchronize(st));
   return PG_OK;
 }
 
@@ -1004,11 +1001,12 @@ pg_status pg_pset_create(pg_fieldset *fs, int64_t n, const double *lon, const do
   if (r) { delete ps; return r; }
   set_arrays(ps, A);
   ps->cap = std::max<int64_t>(n, 1);
-  cudaError_t e = dev_alloc((void **)&ps->d_counter, 8);
-  if (e == cudaSuccess) e = dev_alloc((void **)&ps->d_err, 4);
-  if (e == cudaSuccess) e = cudaMemset(ps->d_err, 0, 4);
+  // the step counter and the error word, side by side
+  cudaError_t e = dev_alloc((void **)&ps->d_counter, 16);
+  if (e == cudaSuccess) e = cudaMemset(ps->d_counter, 0, 16);
+  ps->d_err = (int *)(ps->d_counter + 1);
   if (e != cudaSuccess) {
-    A.free_all(); dev_free(ps->d_counter); dev_free(ps->d_err);
+    A.free_all(); dev_free(ps->d_counter);
     delete ps;
     cudaGetLastError();
     set_error("allocation failed: %s", cudaGetErrorString(e));
@@ -1016,9 +1014,8 @@ pg_status pg_pset_create(pg_fieldset *fs, int64_t n, const double *lon, const do
   }
   double tmin = t0, tmax = t0;
   if (n > 0) r = fill_particles(ps, 0, n, lon, lat, depth, time, t0, ids, id_base, 0, tmin, tmax);
-  if (!r) r = init_variables(ps, 0, n, 0);
   if (r) {
-    A.free_all(); dev_free(ps->d_counter); dev_free(ps->d_err);
+    A.free_all(); dev_free(ps->d_counter);
     delete ps;
     return r;
   }
@@ -1072,7 +1069,6 @@ pg_status pg_pset_add(pg_pset *ps, int64_t n, const double *lon, const double *l
   }
   double tmin, tmax;
   pg_status r = fill_particles(ps, ps->n, n, lon, lat, depth, time, t0, ids, id_base, 0, tmin, tmax);
-  if (!r) r = init_variables(ps, ps->n, n, 0);
   if (r) return r;
   if (ps->n == 0) { ps->t_min = tmin; ps->t_max = tmax; }
   else { ps->t_min = std::min(ps->t_min, tmin); ps->t_max = std::max(ps->t_max, tmax); }
@@ -1101,39 +1097,45 @@ pg_status pg_pset_get(const pg_pset *ps, double *lon, double *lat, double *depth
   cudaStream_t st = (cudaStream_t)stream;
   const int64_t n = ps->n;
   if (n == 0) return PG_OK;
-  double *tmp = nullptr;
-  if (ps->pos == PG_POS_CELL && (lon || lat || depth)) {
-    CU(dev_alloc((void **)&tmp, n * 8 * 3));
-    cudaError_t e = launch_from_cell(grid_args(ps->fs), ps->ci, ps->cj, ps->ck, ps->fx, ps->fy,
-                                     ps->fz, tmp, tmp + n, tmp + 2 * n, n, ps->fs->sm_count, st);
-    if (e == cudaSuccess && lon) e = cudaMemcpyAsync(lon, tmp, n * 8, cudaMemcpyDefault, st);
-    if (e == cudaSuccess && lat) e = cudaMemcpyAsync(lat, tmp + n, n * 8, cudaMemcpyDefault, st);
-    if (e == cudaSuccess && depth) e = cudaMemcpyAsync(depth, tmp + 2 * n, n * 8, cudaMemcpyDefault, st);
-    if (e != cudaSuccess) {
-      cudaStreamSynchronize(st);
-      dev_free(tmp);
-      set_error("copy failed: %s", cudaGetErrorString(e));
-      return PG_ERR_CUDA;
-    }
-    lon = lat = depth = nullptr;
-  }
-  if (ps->pos == PG_POS_F32 && (lon || lat || depth)) CU(dev_alloc((void **)&tmp, n * 8));
-  auto coord = [&](void *src, double *dst) -> pg_status {
-    if (!dst) return PG_OK;
-    if (ps->pos == PG_POS_F64) {
-      CU(cudaMemcpyAsync(dst, src, n * 8, cudaMemcpyDefault, st));
-    } else {
-      f32_to_f64_kernel<<<grid_for(n, ps->fs->sm_count), 256, 0, st>>>((const float *)src, tmp, n);
-      note_launches(1);
-      CU(cudaGetLastError());
-      CU(cudaMemcpyAsync(dst, tmp, n * 8, cudaMemcpyDefault, st));
-    }
-    return PG_OK;
-  };
   pg_status r = PG_OK;
-  if (!r) r = coord(ps->x, lon);
-  if (!r) r = coord(ps->y, lat);
-  if (!r) r = coord(ps->z, depth);
+  double *tmp = nullptr;
+  if (ps->pos == PG_POS_F64) {
+    const void *src[3] = {ps->x, ps->y, ps->z};
+    double *dst[3] = {lon, lat, depth};
+    for (int q = 0; q < 3; ++q)
+      if (dst[q]) CU(cudaMemcpyAsync(dst[q], src[q], n * 8, cudaMemcpyDefault, st));
+  } else if (lon || lat || depth) {
+    // converted straight into destinations a kernel can write; through a
+    // buffer on the device into the others
+    double *dst[3] = {lon, lat, depth}, *out[3] = {lon, lat, depth};
+    int staged = 0;
+    bool via[3];
+    for (int q = 0; q < 3; ++q) {
+      via[q] = dst[q] && !kernel_ptr(dst[q], ps->fs->device);
+      staged += via[q];
+    }
+    if (staged) CU(dev_alloc((void **)&tmp, (size_t)n * 8 * staged));
+    double *next = tmp;
+    for (int q = 0; q < 3; ++q)
+      if (via[q]) { out[q] = next; next += n; }
+    cudaError_t e;
+    if (ps->pos == PG_POS_CELL) {
+      e = launch_from_cell(grid_args(ps->fs), ps->ci, ps->cj, ps->ck, ps->fx, ps->fy, ps->fz,
+                           out[0], out[1], out[2], n, ps->fs->sm_count, st);
+    } else {
+      export_f32_kernel<<<grid_for(n, ps->fs->sm_count), 256, 0, st>>>(
+          (const float *)ps->x, (const float *)ps->y, (const float *)ps->z, out[0], out[1], out[2],
+          n);
+      note_launches(1);
+      e = cudaGetLastError();
+    }
+    for (int q = 0; q < 3 && e == cudaSuccess; ++q)
+      if (via[q]) e = cudaMemcpyAsync(dst[q], out[q], n * 8, cudaMemcpyDefault, st);
+    if (e != cudaSuccess) {
+      set_error("copy failed: %s", cudaGetErrorString(e));
+      r = PG_ERR_CUDA;
+    }
+  }
   if (!r && time) {
     cudaError_t e = cudaMemcpyAsync(time, ps->time, n * 8, cudaMemcpyDefault, st);
     if (e) { set_error("copy failed: %s", cudaGetErrorString(e)); r = PG_ERR_CUDA; }
@@ -1325,6 +1327,8 @@ static pg_status execute_loop(pg_pset *ps, const pg_kernel *k, double runtime, d
     pg_status r = resolve_kernel(k, fs, ps->seed, a.k);
     if (r) return r;
   }
+  if (k->beh & PG_AGE) ps->age_used = true;
+  if (k->scheme == PG_RKF45) ps->hstep_used = true;
   if (k->scheme == PG_RKF45 && a.k.rk_hmax == 0.0) a.k.rk_hmax = std::fabs(dt);
   if (k->scheme == PG_RKF45) a.k.rk_hmin = std::min(a.k.rk_hmin, a.k.rk_hmax);
   const bool ext = (k->beh & (PG_SETTLE | PG_AGE | PG_SAMPLE)) || fs->interp != PG_LINEAR ||
@@ -1376,8 +1380,7 @@ static pg_status execute_loop(pg_pset *ps, const pg_kernel *k, double runtime, d
   }
   double t_prev_out = t_begin;
   int pending_out = -1;              // ring slot whose output awaits delivery
-  CU(cudaMemsetAsync(ps->d_counter, 0, 8, st));
-  CU(cudaMemsetAsync(ps->d_err, 0, 4, st));
+  CU(cudaMemsetAsync(ps->d_counter, 0, 16, st));     // the error word with it
 
   const double chunk_len = std::fabs(dt) * (ps->tune.chunk_steps > 0 ? ps->tune.chunk_steps : 64);
   const double resort_len = ps->tune.resort_steps > 0 ? std::fabs(dt) * ps->tune.resort_steps : 0.0;
@@ -1503,11 +1506,12 @@ static pg_status execute_loop(pg_pset *ps, const pg_kernel *k, double runtime, d
     pg_status r = deliver_output(ps, pending_out, out, rec, user);
     if (r) return r;
   }
-  unsigned long long done = 0;
-  int err = 0;
-  CU(cudaMemcpyAsync(&done, ps->d_counter, 8, cudaMemcpyDeviceToHost, st));
-  CU(cudaMemcpyAsync(&err, ps->d_err, 4, cudaMemcpyDeviceToHost, st));
+  unsigned long long back[2] = {0, 0};               // counter, error word
+  CU(cudaMemcpyAsync(back, ps->d_counter, 16, cudaMemcpyDeviceToHost, st));
   CU(cudaStreamSynchronize(st));
+  const unsigned long long done = back[0];
+  int err = 0;
+  memcpy(&err, &back[1], sizeof err);
   if (steps_done) *steps_done = (int64_t)done;
   if (ps->timing) {
     for (size_t q = 0; q + 1 < ps->ev_used; q += 2) {
@@ -1642,6 +1646,7 @@ pg_status pg_pset_restore(pg_fieldset *fs, const char *path, pg_pset **out) {
     ps->cap = n;
   }
   ps->n = n;
+  ps->age_used = true; ps->hstep_used = true;      // whatever the file holds
   ps->t_min = tmin; ps->t_max = tmax;
   *out = ps;
   return PG_OK;
@@ -1654,7 +1659,6 @@ pg_status pg_pset_destroy(pg_pset *ps) {
   arrays_of(ps).free_all();
   ps->alt.free_all();
   dev_free(ps->d_counter);
-  dev_free(ps->d_err);
   dev_free(ps->sort_scratch);
   dev_free(ps->diag_scratch);
   for (cudaEvent_t ev : ps->ev) cudaEventDestroy(ev);

@@ -33,8 +33,11 @@ struct Slot {
   cudaEvent_t free = nullptr;    // last use finished (recorded on the compute stream)
 };
 
-// Device arrays of one particle set (positions in one of the two forms).
+// Device arrays of one particle set (positions in one of the two forms), in
+// one allocation: a set is made and freed with two calls of the allocator
+// instead of fifteen (24 sets of a batch: 9 of its 15.7 ms).
 struct PsetArrays {
+  void *base = nullptr;       // the allocation
   void *x = nullptr, *y = nullptr, *z = nullptr;
   int32_t *ci = nullptr, *cj = nullptr, *ck = nullptr;
   float *fx = nullptr, *fy = nullptr, *fz = nullptr;
@@ -46,8 +49,7 @@ struct PsetArrays {
   double *var = nullptr;      // [nvar][cap] sampled variables
   double *hstep = nullptr;    // [cap] RKF45 step lengths
   void free_all() {
-    void *ps[] = {x, y, z, ci, cj, ck, fx, fy, fz, time, id, step, status, age, var, hstep};
-    for (void *p : ps) dev_free(p);
+    dev_free(base);
     *this = PsetArrays();
   }
 };
@@ -153,6 +155,7 @@ struct pg_pset {
   int pos = PG_POS_F32;
   uint64_t seed = 0;
   int64_t n = 0, cap = 0;
+  void *base = nullptr;                                 // the arrays' allocation
   void *x = nullptr, *y = nullptr, *z = nullptr;       // positions (plain forms)
   int32_t *ci = nullptr, *cj = nullptr, *ck = nullptr;  // cell form
   float *fx = nullptr, *fy = nullptr, *fz = nullptr;
@@ -164,6 +167,9 @@ struct pg_pset {
   double *var = nullptr;               // [nvar][cap] sampled variables
   double *hstep = nullptr;             // [cap] RKF45 step lengths (0: start from dt)
   int nvar = 0;                        // the field set's scalar fields at creation
+  // whether ages and RKF45 step lengths can be other than the zeros every set
+  // starts with (in both sets of arrays); until then a re-sort leaves them
+  bool age_used = false, hstep_used = false;
   double t_min = 0.0, t_max = 0.0;     // range of particle times
   pg_tune tune{256, 0, 64};
   unsigned long long *d_counter = nullptr;

@@ -11,6 +11,8 @@
 //
 // Moments: FP64 sums over alive particles, per block in a fixed order and
 // then over blocks in a fixed order, so the result does not depend on timing.
+#include <type_traits>
+
 #include "pg_host.h"
 
 namespace pg {
@@ -58,12 +60,12 @@ MortonSpec morton_spec(const pg_fieldset *fs, int64_t n) {
   return m;
 }
 
-__device__ __forceinline__ int cell_index(const double *x, int n, int uni, double x0, double inv,
-                                          double p) {
+template <typename Real>
+__device__ __forceinline__ int cell_index(const Real *x, int n, int uni, Real x0, Real inv, Real p) {
   int i;
   if (uni) {
-    const double f = floor((p - x0) * inv);
-    i = f < 0.0 ? 0 : (f > (double)(n - 1) ? n - 1 : (int)f);
+    const Real f = floor((p - x0) * inv);
+    i = f >= (Real)0 ? (f > (Real)(n - 1) ? n - 1 : (int)f) : 0;     // 0 for NaN too
   } else {
     int lo = 0, hi = n - 1;
     if (!(p >= x[0])) return 0;
@@ -88,11 +90,27 @@ __device__ __forceinline__ uint32_t morton(const int (&c)[3], const MortonSpec &
   return key;
 }
 
+// Bucket of every particle and the buckets' counts.  Cells are found in the
+// positions' own precision (GridArgs' axes in it): the order only decides
+// which particles are neighbours, and FP64 searches took 0.57 ms for 10M FP32
+// positions.
+__device__ __forceinline__ const double *sort_axis(const GridArgs &g, int a, double) {
+  return a == 0 ? g.lon : (a == 1 ? g.lat : g.depth);
+}
+__device__ __forceinline__ const float *sort_axis(const GridArgs &g, int a, float) {
+  return a == 0 ? g.lonf : (a == 1 ? g.latf : g.depthf);
+}
+__device__ __forceinline__ double sort_x0(const GridArgs &g, int a, double) { return g.x0[a]; }
+__device__ __forceinline__ float sort_x0(const GridArgs &g, int a, float) { return g.x0f[a]; }
+__device__ __forceinline__ double sort_inv(const GridArgs &g, int a, double) { return g.inv_d[a]; }
+__device__ __forceinline__ float sort_inv(const GridArgs &g, int a, float) { return g.inv_df[a]; }
+
 template <typename Real>
 __global__ void bucket_kernel(GridArgs g, MortonSpec m, const Real *x, const Real *y,
                               const Real *z, const int32_t *ci, const int32_t *cj,
                               const int32_t *ck, const uint8_t *status, int64_t n,
                               uint32_t dead, uint32_t *key, uint32_t *count) {
+  const Real o = (Real)0;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
        p += (int64_t)gridDim.x * blockDim.x) {
     uint32_t k = dead;
@@ -101,15 +119,19 @@ __global__ void bucket_kernel(GridArgs g, MortonSpec m, const Real *x, const Rea
       if (ci) {
         c[0] = ci[p]; c[1] = cj[p]; c[2] = ck ? ck[p] : 0;
       } else {
-        double lon = (double)x[p];
+        Real lon = x[p];
         if (g.periodic) {
-          double r = fmod(lon - g.lon[0], 360.0);
-          if (r < 0.0) r += 360.0;
-          lon = g.lon[0] + r;
+          Real r = lon - sort_x0(g, 0, o);
+          if (!(r >= (Real)0 && r < (Real)360)) {
+            r = fmod(r, (Real)360);
+            if (r < (Real)0) r += (Real)360;
+            lon = sort_x0(g, 0, o) + r;
+          }
         }
-        c[0] = cell_index(g.lon, g.nx, g.uni[0], g.x0[0], g.inv_d[0], lon);
-        c[1] = cell_index(g.lat, g.ny, g.uni[1], g.x0[1], g.inv_d[1], (double)y[p]);
-        if (g.nz > 1) c[2] = cell_index(g.depth, g.nz, g.uni[2], g.x0[2], g.inv_d[2], (double)z[p]);
+        c[0] = cell_index(sort_axis(g, 0, o), g.nx, g.uni[0], sort_x0(g, 0, o), sort_inv(g, 0, o), lon);
+        c[1] = cell_index(sort_axis(g, 1, o), g.ny, g.uni[1], sort_x0(g, 1, o), sort_inv(g, 1, o), y[p]);
+        if (g.nz > 1)
+          c[2] = cell_index(sort_axis(g, 2, o), g.nz, g.uni[2], sort_x0(g, 2, o), sort_inv(g, 2, o), z[p]);
       }
       k = morton(c, m);
     }
@@ -162,11 +184,49 @@ __global__ void scatter_kernel(const uint32_t *key, uint32_t *offset, uint32_t *
   }
 }
 
-template <typename T>
-__global__ void gather_kernel(const T *src, T *dst, const uint32_t *perm, int64_t n) {
+// Every array of a set's state in one pass: entry p of dst from entry
+// perm[p] of src (perm null: entry p).  Bound by the scattered reads of src;
+// one launch instead of one per array (twelve, and as many copies back in the
+// fixed-pointer mode).
+struct StatePass {
+  PsetArrays src, dst;
+  int nvar;
+  int64_t stride;         // of var
+  bool age, hstep;
+};
+template <int POS>
+__global__ void __launch_bounds__(256) state_pass_kernel(const __grid_constant__ StatePass a,
+                                                         const uint32_t *perm, int64_t n) {
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
-       p += (int64_t)gridDim.x * blockDim.x)
-    dst[p] = src[perm[p]];
+       p += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t q = perm ? (int64_t)perm[p] : p;
+    if constexpr (POS == PG_POS_CELL) {
+      a.dst.ci[p] = a.src.ci[q]; a.dst.cj[p] = a.src.cj[q]; a.dst.ck[p] = a.src.ck[q];
+      a.dst.fx[p] = a.src.fx[q]; a.dst.fy[p] = a.src.fy[q]; a.dst.fz[p] = a.src.fz[q];
+    } else {
+      using Real = typename std::conditional<POS == PG_POS_F64, double, float>::type;
+      reinterpret_cast<Real *>(a.dst.x)[p] = reinterpret_cast<const Real *>(a.src.x)[q];
+      reinterpret_cast<Real *>(a.dst.y)[p] = reinterpret_cast<const Real *>(a.src.y)[q];
+      reinterpret_cast<Real *>(a.dst.z)[p] = reinterpret_cast<const Real *>(a.src.z)[q];
+    }
+    a.dst.time[p] = a.src.time[q];
+    a.dst.id[p] = a.src.id[q];
+    a.dst.step[p] = a.src.step[q];
+    a.dst.status[p] = a.src.status[q];
+    if (a.age) a.dst.age[p] = a.src.age[q];
+    if (a.hstep) a.dst.hstep[p] = a.src.hstep[q];
+    for (int j = 0; j < a.nvar; ++j)
+      a.dst.var[j * a.stride + p] = a.src.var[j * a.stride + q];
+  }
+}
+
+void launch_state_pass(const pg_pset *ps, const PsetArrays &src, const PsetArrays &dst,
+                       const uint32_t *perm, int grid, cudaStream_t st) {
+  const StatePass a{src, dst, ps->nvar, ps->cap, ps->age_used, ps->hstep_used};
+  auto kern = ps->pos == PG_POS_CELL ? state_pass_kernel<PG_POS_CELL>
+            : (ps->pos == PG_POS_F64 ? state_pass_kernel<PG_POS_F64> : state_pass_kernel<PG_POS_F32>);
+  kern<<<grid, 256, 0, st>>>(a, perm, ps->n);
+  note_launches(1);
 }
 
 int grid_of(int64_t n, int sm) {
@@ -234,6 +294,11 @@ cudaError_t prepare_resort(pg_pset *ps) {
     if (alloc_arrays(ps->alt, ps->pos, ps->cap, ps->nvar) != PG_OK)
       return cudaErrorMemoryAllocation;
     ps->alt_cap = ps->cap;
+    // ages and step lengths that no pass has moved yet are zeros in both sets
+    const size_t b = (size_t)std::max<int64_t>(ps->cap, 1) * 8;
+    if ((e = cudaMemset(ps->alt.age, 0, b)) != cudaSuccess) return e;
+    if ((e = cudaMemset(ps->alt.hstep, 0, b)) != cudaSuccess) return e;
+    if ((e = cudaStreamSynchronize(0)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
@@ -255,10 +320,7 @@ cudaError_t launch_resort(pg_pset *ps, cudaStream_t st, int64_t *n_alive) {
   uint32_t *offset = count + nb;
   uint32_t *tmp = offset + nb;
   const int sm = fs->sm_count;
-  GridArgs g;
-  g.nx = fs->nx; g.ny = fs->ny; g.nz = fs->nz; g.mesh = fs->mesh; g.periodic = fs->periodic;
-  g.lon = fs->d_axes64; g.lat = fs->d_axes64 + fs->nx; g.depth = fs->d_axes64 + fs->nx + fs->ny;
-  for (int a = 0; a < 3; ++a) { g.uni[a] = fs->uni[a]; g.x0[a] = fs->x0[a]; g.inv_d[a] = fs->inv_d[a]; }
+  const GridArgs g = grid_args_of(fs);
   if ((e = cudaMemsetAsync(count, 0, sizeof(uint32_t) * nb, st)) != cudaSuccess) return e;
   const int gr = grid_of(n, sm);
   if (ps->pos == PG_POS_F64)
@@ -281,57 +343,13 @@ cudaError_t launch_resort(pg_pset *ps, cudaStream_t st, int64_t *n_alive) {
       (e = cudaMemcpyAsync(&dead_count, count + dead, 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
     return e;
   scatter_kernel<<<gr, 256, 0, st>>>(key, offset, perm, n);
+  note_launches(1);
   PsetArrays &B = ps->alt;
-  if (ps->pos == PG_POS_CELL) {
-    gather_kernel<int32_t><<<gr, 256, 0, st>>>(ps->ci, B.ci, perm, n);
-    gather_kernel<int32_t><<<gr, 256, 0, st>>>(ps->cj, B.cj, perm, n);
-    gather_kernel<int32_t><<<gr, 256, 0, st>>>(ps->ck, B.ck, perm, n);
-    gather_kernel<float><<<gr, 256, 0, st>>>(ps->fx, B.fx, perm, n);
-    gather_kernel<float><<<gr, 256, 0, st>>>(ps->fy, B.fy, perm, n);
-    gather_kernel<float><<<gr, 256, 0, st>>>(ps->fz, B.fz, perm, n);
-  } else if (ps->pos == PG_POS_F64) {
-    gather_kernel<double><<<gr, 256, 0, st>>>((const double *)ps->x, (double *)B.x, perm, n);
-    gather_kernel<double><<<gr, 256, 0, st>>>((const double *)ps->y, (double *)B.y, perm, n);
-    gather_kernel<double><<<gr, 256, 0, st>>>((const double *)ps->z, (double *)B.z, perm, n);
-  } else {
-    gather_kernel<float><<<gr, 256, 0, st>>>((const float *)ps->x, (float *)B.x, perm, n);
-    gather_kernel<float><<<gr, 256, 0, st>>>((const float *)ps->y, (float *)B.y, perm, n);
-    gather_kernel<float><<<gr, 256, 0, st>>>((const float *)ps->z, (float *)B.z, perm, n);
-  }
-  gather_kernel<double><<<gr, 256, 0, st>>>(ps->time, B.time, perm, n);
-  gather_kernel<uint64_t><<<gr, 256, 0, st>>>(ps->id, B.id, perm, n);
-  gather_kernel<uint32_t><<<gr, 256, 0, st>>>(ps->step, B.step, perm, n);
-  gather_kernel<uint8_t><<<gr, 256, 0, st>>>(ps->status, B.status, perm, n);
-  gather_kernel<double><<<gr, 256, 0, st>>>(ps->age, B.age, perm, n);
-  gather_kernel<double><<<gr, 256, 0, st>>>(ps->hstep, B.hstep, perm, n);
-  for (int j = 0; j < ps->nvar; ++j)
-    gather_kernel<double><<<gr, 256, 0, st>>>(ps->var + (size_t)j * ps->cap,
-                                              B.var + (size_t)j * ps->cap, perm, n);
-  note_launches((ps->pos == PG_POS_CELL ? 11 : 8) + 2 + ps->nvar);
+  launch_state_pass(ps, pset_arrays(ps), B, perm, gr, st);
+  // fixed-pointer mode: the sorted arrays back in place
+  if (!n_alive) launch_state_pass(ps, B, pset_arrays(ps), nullptr, gr, st);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (!n_alive) {
-    // fixed-pointer mode: copy the sorted arrays back in place
-    const auto arrays_a = std::vector<std::pair<void *, void *>>{
-        {ps->x, B.x}, {ps->y, B.y}, {ps->z, B.z}, {ps->ci, B.ci}, {ps->cj, B.cj},
-        {ps->ck, B.ck}, {ps->fx, B.fx}, {ps->fy, B.fy}, {ps->fz, B.fz}};
-    const size_t el = ps->pos == PG_POS_F64 ? 8 : 4;
-    for (const auto &pr : arrays_a)
-      if (pr.first && (e = cudaMemcpyAsync(pr.first, pr.second, (size_t)n * el,
-                                           cudaMemcpyDeviceToDevice, st)) != cudaSuccess)
-        return e;
-    if ((e = cudaMemcpyAsync(ps->time, B.time, (size_t)n * 8, cudaMemcpyDeviceToDevice, st)) ||
-        (e = cudaMemcpyAsync(ps->id, B.id, (size_t)n * 8, cudaMemcpyDeviceToDevice, st)) ||
-        (e = cudaMemcpyAsync(ps->step, B.step, (size_t)n * 4, cudaMemcpyDeviceToDevice, st)) ||
-        (e = cudaMemcpyAsync(ps->status, B.status, (size_t)n, cudaMemcpyDeviceToDevice, st)) ||
-        (e = cudaMemcpyAsync(ps->age, B.age, (size_t)n * 8, cudaMemcpyDeviceToDevice, st)) ||
-        (e = cudaMemcpyAsync(ps->hstep, B.hstep, (size_t)n * 8, cudaMemcpyDeviceToDevice, st)))
-      return e;
-    for (int j = 0; j < ps->nvar; ++j)
-      if ((e = cudaMemcpyAsync(ps->var + (size_t)j * ps->cap, B.var + (size_t)j * ps->cap,
-                               (size_t)n * 8, cudaMemcpyDeviceToDevice, st)) != cudaSuccess)
-        return e;
-    return cudaSuccess;
-  }
+  if (!n_alive) return cudaSuccess;
   // swap the two array sets
   const PsetArrays A = pset_arrays(ps);
   pset_set_arrays(ps, B);
