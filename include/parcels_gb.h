@@ -149,10 +149,12 @@ typedef struct {
 
 /* Tuning of the time loop.  Zero fields take defaults. */
 typedef struct {
-    int block;          /* threads per block of the advection kernel (default 256)  */
+    int block;          /* threads per block of the advection kernel (default 256;  */
+                        /* fewer in a launch that would leave multiprocessors idle)  */
     int resort_steps;   /* Morton re-sort before the first launch of an execute and
                            every this many steps (0: never)                          */
-    int chunk_steps;    /* at most this many steps per kernel launch (default 64)    */
+    int chunk_steps;    /* at most this many steps per kernel launch (0: chosen by   */
+                        /* the library; results do not depend on it)                 */
 } pg_tune;
 
 /* Snapshot source for streamed fields (the counterpart of advancing the

@@ -129,9 +129,9 @@ template <typename Store, int NF, bool D3, int GEO>
 // third of the corner values: at most 85 registers, six 128-thread blocks
 // (24 warps) per SM, measured faster than five or four.
 __global__ void __launch_bounds__(D3 ? 256 : 128, D3 ? 2 : 6) advect_cell_kernel(StepArgs a) {
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t p = lane_particle(a.lanes);
   unsigned long long done = 0;
-  if (p < a.p.n && a.p.status[p] == 0) {
+  if (p >= 0 && p < a.p.n && a.p.status[p] == 0) {
     CellState s;
     s.i = a.p.ci[p]; s.j = a.p.cj[p]; s.x = a.p.fx[p]; s.y = a.p.fy[p];
     if (D3) { s.k = a.p.ck[p]; s.z = a.p.fz[p]; } else { s.k = 0; s.z = 0.f; }

@@ -10,10 +10,10 @@ template <typename Store>
 static cudaError_t launch_f64(const StepArgs &a, int block, cudaStream_t st) {
   if (a.p.n == 0) return cudaSuccess;
   if (a.f.nf == 3)
-    return launch_clamped<advect_plain_kernel<double, Store, 3, true, GEO_ANY>>(a, block, st);
+    return launch_clamped<advect_plain_kernel<double, Store, 3, true, GEO_ANY>>(a, block, st, kSparseWarps64);
   if (a.g.nz > 1)
-    return launch_clamped<advect_plain_kernel<double, Store, 2, true, GEO_ANY>>(a, block, st);
-  return launch_clamped<advect_plain_kernel<double, Store, 2, false, GEO_ANY>>(a, block, st);
+    return launch_clamped<advect_plain_kernel<double, Store, 2, true, GEO_ANY>>(a, block, st, kSparseWarps64);
+  return launch_clamped<advect_plain_kernel<double, Store, 2, false, GEO_ANY>>(a, block, st, kSparseWarps64);
 }
 
 cudaError_t launch_advect_f64(const StepArgs &a, int storage, int block, cudaStream_t st) {

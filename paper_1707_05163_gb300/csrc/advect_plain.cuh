@@ -658,9 +658,9 @@ template <typename Real, typename Store, int NF, bool D3, int GEO, bool EXT = fa
 __global__ void __launch_bounds__(sizeof(Real) == 4 && !D3 ? 128 : 256,
                                   sizeof(Real) == 4 ? (D3 ? 2 : (EXT ? 6 : 7)) : 1)
     advect_plain_kernel(StepArgs a) {
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t p = lane_particle(a.lanes);
   unsigned long long done = 0;
-  if (p < a.p.n && a.p.status[p] == 0) done = advance_particle<EXT, Real, Store, NF, D3, GEO>(a, p);
+  if (p >= 0 && p < a.p.n && a.p.status[p] == 0) done = advance_particle<EXT, Real, Store, NF, D3, GEO>(a, p);
   count_steps(done, a.steps_done);
 }
 

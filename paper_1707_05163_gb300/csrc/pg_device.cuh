@@ -108,7 +108,16 @@ struct StepArgs {
   double t_clip;                    // RKF45 steps land on this time (next output) and t_end
   unsigned long long *steps_done;   // particle-steps taken (device counter)
   int *err;                         // first DevErr recorded (device word)
+  int lanes = 32;                   // particles per warp (lane_particle)
 };
+
+// The particle of this thread: warp w holds particles w * lanes .. + lanes in
+// its first lanes; the others have none (-1).
+__device__ __forceinline__ int64_t lane_particle(int lanes) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (lanes == 32) return t;
+  return (int)(t & 31) < lanes ? (t >> 5) * lanes + (t & 31) : -1;
+}
 
 // ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds of two

@@ -171,7 +171,7 @@ struct pg_pset {
   // starts with (in both sets of arrays); until then a re-sort leaves them
   bool age_used = false, hstep_used = false;
   double t_min = 0.0, t_max = 0.0;     // range of particle times
-  pg_tune tune{256, 0, 64};
+  pg_tune tune{256, 0, 0};             // chunk_steps 0: chosen per execute
   unsigned long long *d_counter = nullptr;
   int *d_err = nullptr;
   // re-sort: second set of arrays (same capacity) and scratch, on first use
@@ -262,22 +262,33 @@ inline int geo_of(const GridArgs &g) {
   return g.mesh != 1 ? GEO_FLAT : (g.periodic ? GEO_SPH_PER : GEO_SPH);
 }
 
-// Block size of a launch over n particles: the given one, halved (to a warp
-// at least) while the blocks would not give every multiprocessor two.  A set
-// that small runs at the latency of its threads' chains of steps, or, in
-// FP64, at the pipe's rate on the multiprocessors that have a block: 10,000
-// FP64 particles in 40 blocks of 256 used 40 of 152 (a 64-step launch of the
-// gyre 1.32 ms, in 313 blocks of 32 a quarter of that).
-inline int spread_block(int64_t n, int block, int sms) {
-  while (block >= 64 && block % 64 == 0 && n <= (int64_t)block * (2 * sms - 1)) block /= 2;
-  return block;
+// Shape of a launch over n particles of a set that does not fill the chip.
+// Block: the given one, halved (to a warp at least) while the blocks would
+// not give every multiprocessor two -- 10,000 FP64 particles in 40 blocks of
+// 256 used 40 of 152.  Lanes: 32 particles per warp, fewer, in powers of two,
+// while the warps are at most `sparse` per multiprocessor: such a launch
+// lasts as long as its slowest warp's chain of stages, and a warp takes the
+// slow path of a stage (a cell change: searches and dependent loads, four
+// times the rest of the stage) whenever one of its lanes does.
+// FP64 (one pipe per multiprocessor, 16 clocks a warp instruction whatever
+// its lanes): one warp per multiprocessor (10,000 particles: 8.4 ms with 32
+// lanes, 10.5 ms with 16).
+constexpr int kSparseWarps = 8, kSparseWarps64 = 1;
+inline void launch_shape(int64_t n, int block, int sms, int sparse, int &b, int &lanes) {
+  b = block;
+  lanes = 32;
+  if (sms <= 0) return;
+  while (lanes > 1 && (n + lanes / 2 - 1) / (lanes / 2) <= (int64_t)sms * sparse) lanes /= 2;
+  const int64_t threads = (n + lanes - 1) / lanes * 32;
+  while (b >= 64 && b % 64 == 0 && threads <= (int64_t)b * (2 * sms - 1)) b /= 2;
 }
 
 // Launch a chunk kernel over a.p.n particles, one thread each.  The block
 // size is clamped to what the kernel's register use allows (queried once per
-// kernel) and spread over the multiprocessors.
+// kernel).
 template <void (*Kernel)(StepArgs)>
-inline cudaError_t launch_clamped(const StepArgs &a, int block, cudaStream_t st) {
+inline cudaError_t launch_clamped(const StepArgs &a, int block, cudaStream_t st,
+                                  int sparse = kSparseWarps) {
   static int max_threads = 0;
   static int sms = 0;
   if (max_threads == 0) {
@@ -290,9 +301,12 @@ inline cudaError_t launch_clamped(const StepArgs &a, int block, cudaStream_t st)
     sms = q;
     max_threads = at.maxThreadsPerBlock;
   }
-  const int b = spread_block(a.p.n, block > max_threads ? (max_threads / 32) * 32 : block, sms);
-  const int64_t grid = (a.p.n + b - 1) / b;
-  Kernel<<<(unsigned)grid, b, 0, st>>>(a);
+  StepArgs s = a;
+  int b;
+  launch_shape(a.p.n, block > max_threads ? (max_threads / 32) * 32 : block, sms, sparse, b, s.lanes);
+  const int64_t threads = (a.p.n + s.lanes - 1) / s.lanes * 32;
+  const int64_t grid = (threads + b - 1) / b;
+  Kernel<<<(unsigned)grid, b, 0, st>>>(s);
   note_launches(1);
   return cudaGetLastError();
 }
