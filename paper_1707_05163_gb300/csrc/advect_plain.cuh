@@ -533,10 +533,12 @@ __device__ __forceinline__ void sample_variables(const A &a, int64_t p, double l
   }
 }
 
+enum : int { EXT_BEHAVIOURS = 1, EXT_RKF45 = 2 };
+
 // The chunk kernel: each thread advances one particle while its time is
 // before t_stop and t_end (in the direction of dt), shortening only the step
 // that lands on t_end.  Returns the number of steps taken.
-template <bool EXT, typename Real, typename Store, int NF, bool D3, int GEO, class A>
+template <int EXT, typename Real, typename Store, int NF, bool D3, int GEO, class A>
 __device__ __forceinline__ unsigned long long advance_particle(const A &a, int64_t p) {
   constexpr bool X = EXT || sizeof(Real) == 8;
   unsigned long long done = 0;
@@ -559,11 +561,12 @@ __device__ __forceinline__ unsigned long long advance_particle(const A &a, int64
     Clock ck;
     ck.dt = a.dt; ck.k = 0; ck.d = 0.f;
     bool adaptive = false;
-    if constexpr (X) adaptive = a.k.scheme == 2;
+    if constexpr (sizeof(Real) == 8) adaptive = a.k.scheme == 2;
+    else adaptive = EXT == EXT_RKF45;
     if (adaptive) {
       if constexpr (X) {
         double hp = a.p.hstep[p];
-        done = rkf45_steps<EXT>(a, c, lon, lat, dep, t, stp, hp, age, st, idp);
+        done = rkf45_steps<(EXT != 0)>(a, c, lon, lat, dep, t, stp, hp, age, st, idp);
         a.p.hstep[p] = hp;
       }
     } else if constexpr (sizeof(Real) == 8) {
@@ -575,7 +578,7 @@ __device__ __forceinline__ unsigned long long advance_particle(const A &a, int64
         const double left = a.t_end - t;
         if (fwd ? left < h : left > h) h = left;
         ck.t = t;
-        const int r = step_one<EXT>(a, c, ck, lon, lat, dep, (Real)h, h, age, idp, stp);
+        const int r = step_one<(EXT != 0)>(a, c, ck, lon, lat, dep, (Real)h, h, age, idp, stp);
         if (r == STATUS_DELETED) {      // taken, then deleted by the age behaviour
           t = t + h;
           ++stp;
@@ -605,7 +608,7 @@ __device__ __forceinline__ unsigned long long advance_particle(const A &a, int64
       for (; k < n; ++k) {
         ck.k = k;
         const float h = (k == n - 1) ? hlf : hf;
-        const int r = step_one<EXT>(a, c, ck, lon, lat, dep, (Real)h,
+        const int r = step_one<(EXT != 0)>(a, c, ck, lon, lat, dep, (Real)h,
                                     (k == n - 1) ? hlast : a.dt, age, idp, stp);
         if (r > 0) {
           if (X && r == STATUS_DELETED) {   // taken, then deleted by the age behaviour
@@ -651,10 +654,10 @@ __device__ __forceinline__ void count_steps(unsigned long long done, unsigned lo
 // on the 1/12-degree workload, a few spilled words); with the worked
 // example's behaviours, six.
 //
-// EXT = true: the FP32 kernel with the worked example's behaviours (settle,
-// age, sampled variables) and nearest-neighbour interpolation; the FP64
-// kernel always has them.
-template <typename Real, typename Store, int NF, bool D3, int GEO, bool EXT = false>
+// EXT (FP32): EXT_BEHAVIOURS adds the worked example's behaviours (settle, age,
+// sampled variables) and nearest-neighbour interpolation to the fixed steps,
+// EXT_RKF45 has them with the adaptive steps; the FP64 kernel always has all.
+template <typename Real, typename Store, int NF, bool D3, int GEO, int EXT = 0>
 __global__ void __launch_bounds__(sizeof(Real) == 4 && !D3 ? 128 : 256,
                                   sizeof(Real) == 4 ? (D3 ? 2 : (EXT ? 6 : 7)) : 1)
     advect_plain_kernel(StepArgs a) {
@@ -723,7 +726,7 @@ __global__ void __launch_bounds__(256, 2) advect_batch_kernel(const __grid_const
     if (t >= b.ntiles) break;
     const BatchStep v{b.g, b.f, sk, sp, sdt, b.t_stop, st_end, b.steps_done, b.err};
     const int64_t p = (int64_t)b.tiles[t].y + threadIdx.x;
-    if (p < sp.n && sp.status[p] == 0) done += advance_particle<false, float, Store, NF, D3, GEO>(v, p);
+    if (p < sp.n && sp.status[p] == 0) done += advance_particle<0, float, Store, NF, D3, GEO | CORNERS_SINGLE>(v, p);
     __syncthreads();
   }
   count_steps(done, b.steps_done);

@@ -89,14 +89,17 @@ struct PartArgs {
 // the per-stage mesh and wrap tests cost nothing.  A periodic zonal boundary
 // needs a spherical mesh, so these three kinds cover every field set.
 enum : int { GEO_ANY = 0, GEO_FLAT = 1, GEO_SPH = 2, GEO_SPH_PER = 3 };
+// Added to the geometry: the kernel keeps its corner values one by one rather
+// than in pairs (Sampler).
+enum : int { GEO_MASK = 3, CORNERS_SINGLE = 4 };
 
 template <int GEO> __device__ __forceinline__ bool is_sph(const GridArgs &g) {
-  if constexpr (GEO == GEO_ANY) return g.mesh == 1;
-  else return GEO != GEO_FLAT;
+  if constexpr ((GEO & GEO_MASK) == GEO_ANY) return g.mesh == 1;
+  else return (GEO & GEO_MASK) != GEO_FLAT;
 }
 template <int GEO> __device__ __forceinline__ bool is_per(const GridArgs &g) {
-  if constexpr (GEO == GEO_ANY) return g.periodic != 0;
-  else return GEO == GEO_SPH_PER;
+  if constexpr ((GEO & GEO_MASK) == GEO_ANY) return g.periodic != 0;
+  else return (GEO & GEO_MASK) == GEO_SPH_PER;
 }
 
 struct StepArgs {
