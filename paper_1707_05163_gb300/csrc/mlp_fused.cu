@@ -315,12 +315,25 @@ __device__ __forceinline__ void store_input_row(uint8_t *dst, int r, const uint3
 // kernel they took 46k clocks per 128-row tile, four times the network's.
 __global__ void __launch_bounds__(128) pack_features_kernel(const __grid_constant__ SurrogateStepIO io,
                                                             int64_t rows, uint8_t *out) {
-  const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  // Particles of a set mostly share their time, and its interval costs some
+  // fifty FP64 instructions of 16 clocks of the multiprocessor each: the first
+  // warp finds that of the block's first particle for all that share it.
+  __shared__ SurInterval first;
+  const int64_t m0 = (int64_t)blockIdx.x * blockDim.x, m = m0 + threadIdx.x;
+  const double t0 = m0 < io.n ? io.time[m0] : 0.0;
+  if (threadIdx.x < 32) {
+    const SurInterval v = surrogate_interval(io.f, t0);
+    if (threadIdx.x == 0) first = v;
+  }
+  __syncthreads();
   if (m >= rows) return;
   float o[kSurFeat];
   bool ok = false;
   if (m < io.n && io.status[m] == 0) {
-    const int e = surrogate_features(io.g, io.f, io.lon[m], io.lat[m], io.dep[m], io.time[m], o);
+    const double t = io.time[m];
+    const SurInterval iv = __double_as_longlong(t) == __double_as_longlong(t0)
+                               ? first : surrogate_interval(io.f, t);
+    const int e = surrogate_features(io.g, io.f, io.lon[m], io.lat[m], io.dep[m], iv, o);
     if (e) atomicCAS(io.ferr, 0, e);
     else ok = true;
   }

@@ -11,8 +11,6 @@
 //
 // Moments: FP64 sums over alive particles, per block in a fixed order and
 // then over blocks in a fixed order, so the result does not depend on timing.
-#include <type_traits>
-
 #include "pg_host.h"
 
 namespace pg {
@@ -184,49 +182,76 @@ __global__ void scatter_kernel(const uint32_t *key, uint32_t *offset, uint32_t *
   }
 }
 
-// Every array of a set's state in one pass: entry p of dst from entry
-// perm[p] of src (perm null: entry p).  Bound by the scattered reads of src;
-// one launch instead of one per array (twelve, and as many copies back in the
-// fixed-pointer mode).
+// Arrays of a set's state moved in one pass: entry p of dst from entry perm[p]
+// of src (perm null: entry p).  A permuted pass is bound by its scattered
+// reads, so arrays share a pass only while they stay in L2 together: the
+// passes of a set of up to a million particles take them all (one launch in
+// place of twelve); of 10M particles, all at once were 1.03 ms, and passes
+// of at most kPassBytes 0.5 ms.
+constexpr int kPassArrays = 8;
+constexpr size_t kPassBytes = (size_t)48 << 20;
 struct StatePass {
-  PsetArrays src, dst;
-  int nvar;
-  int64_t stride;         // of var
-  bool age, hstep;
+  const void *src[kPassArrays];
+  void *dst[kPassArrays];
+  int el[kPassArrays];      // 8, 4 or 1 bytes
+  int n = 0;
 };
-template <int POS>
 __global__ void __launch_bounds__(256) state_pass_kernel(const __grid_constant__ StatePass a,
                                                          const uint32_t *perm, int64_t n) {
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
        p += (int64_t)gridDim.x * blockDim.x) {
     const int64_t q = perm ? (int64_t)perm[p] : p;
-    if constexpr (POS == PG_POS_CELL) {
-      a.dst.ci[p] = a.src.ci[q]; a.dst.cj[p] = a.src.cj[q]; a.dst.ck[p] = a.src.ck[q];
-      a.dst.fx[p] = a.src.fx[q]; a.dst.fy[p] = a.src.fy[q]; a.dst.fz[p] = a.src.fz[q];
-    } else {
-      using Real = typename std::conditional<POS == PG_POS_F64, double, float>::type;
-      reinterpret_cast<Real *>(a.dst.x)[p] = reinterpret_cast<const Real *>(a.src.x)[q];
-      reinterpret_cast<Real *>(a.dst.y)[p] = reinterpret_cast<const Real *>(a.src.y)[q];
-      reinterpret_cast<Real *>(a.dst.z)[p] = reinterpret_cast<const Real *>(a.src.z)[q];
-    }
-    a.dst.time[p] = a.src.time[q];
-    a.dst.id[p] = a.src.id[q];
-    a.dst.step[p] = a.src.step[q];
-    a.dst.status[p] = a.src.status[q];
-    if (a.age) a.dst.age[p] = a.src.age[q];
-    if (a.hstep) a.dst.hstep[p] = a.src.hstep[q];
-    for (int j = 0; j < a.nvar; ++j)
-      a.dst.var[j * a.stride + p] = a.src.var[j * a.stride + q];
+    unsigned long long v[kPassArrays];
+#pragma unroll
+    for (int j = 0; j < kPassArrays; ++j)
+      if (j < a.n)
+        v[j] = a.el[j] == 8   ? reinterpret_cast<const unsigned long long *>(a.src[j])[q]
+               : a.el[j] == 4 ? reinterpret_cast<const uint32_t *>(a.src[j])[q]
+                              : reinterpret_cast<const uint8_t *>(a.src[j])[q];
+#pragma unroll
+    for (int j = 0; j < kPassArrays; ++j)
+      if (j < a.n) {
+        if (a.el[j] == 8) reinterpret_cast<unsigned long long *>(a.dst[j])[p] = v[j];
+        else if (a.el[j] == 4) reinterpret_cast<uint32_t *>(a.dst[j])[p] = (uint32_t)v[j];
+        else reinterpret_cast<uint8_t *>(a.dst[j])[p] = (uint8_t)v[j];
+      }
   }
 }
 
 void launch_state_pass(const pg_pset *ps, const PsetArrays &src, const PsetArrays &dst,
                        const uint32_t *perm, int grid, cudaStream_t st) {
-  const StatePass a{src, dst, ps->nvar, ps->cap, ps->age_used, ps->hstep_used};
-  auto kern = ps->pos == PG_POS_CELL ? state_pass_kernel<PG_POS_CELL>
-            : (ps->pos == PG_POS_F64 ? state_pass_kernel<PG_POS_F64> : state_pass_kernel<PG_POS_F32>);
-  kern<<<grid, 256, 0, st>>>(a, perm, ps->n);
-  note_launches(1);
+  StatePass a;
+  size_t bytes = 0;
+  auto flush = [&]() {
+    if (a.n == 0) return;
+    state_pass_kernel<<<grid, 256, 0, st>>>(a, perm, ps->n);
+    note_launches(1);
+    a.n = 0;
+    bytes = 0;
+  };
+  auto move = [&](const void *s, void *d, int el) {
+    const size_t b = (size_t)ps->n * el;
+    if (a.n == kPassArrays || (perm && a.n > 0 && bytes + b > kPassBytes)) flush();
+    a.src[a.n] = s; a.dst[a.n] = d; a.el[a.n] = el;
+    ++a.n;
+    bytes += b;
+  };
+  if (ps->pos == PG_POS_CELL) {
+    move(src.ci, dst.ci, 4); move(src.cj, dst.cj, 4); move(src.ck, dst.ck, 4);
+    move(src.fx, dst.fx, 4); move(src.fy, dst.fy, 4); move(src.fz, dst.fz, 4);
+  } else {
+    const int el = (int)pos_elem(ps->pos);
+    move(src.x, dst.x, el); move(src.y, dst.y, el); move(src.z, dst.z, el);
+  }
+  move(src.step, dst.step, 4);
+  move(src.status, dst.status, 1);
+  move(src.time, dst.time, 8);
+  move(src.id, dst.id, 8);
+  if (ps->age_used) move(src.age, dst.age, 8);
+  if (ps->hstep_used) move(src.hstep, dst.hstep, 8);
+  for (int j = 0; j < ps->nvar; ++j)
+    move(src.var + (size_t)j * ps->cap, dst.var + (size_t)j * ps->cap, 8);
+  flush();
 }
 
 int grid_of(int64_t n, int sm) {

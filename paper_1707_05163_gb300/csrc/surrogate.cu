@@ -37,7 +37,8 @@ __global__ void features_kernel(GridArgs g, FieldArgs f, const float *lon, const
       for (int q = 0; q < kFeat; ++q) o[q] = 0.f;
       continue;
     }
-    const int r = surrogate_features(g, f, lon[p], lat[p], dep[p], time[p], v);
+    const int r = surrogate_features(g, f, lon[p], lat[p], dep[p],
+                                     surrogate_interval(f, time[p]), v);
     if (r) {
       atomicCAS(err, 0, r);
       continue;

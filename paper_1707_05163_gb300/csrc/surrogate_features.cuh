@@ -27,12 +27,35 @@ __device__ __forceinline__ float sur_lerp(float a, float b, float w) {
   return __fadd_rn(a, __fmul_rn(__fsub_rn(b, a), w));
 }
 
+// Snapshots, weight and phase of the period at a time.  err: a device error
+// code (time outside the field), or 0.
+struct SurInterval {
+  int s0 = 0, s1 = 0, err = 0;
+  float tau = 0.f, phase = 0.f;
+};
+__device__ __forceinline__ SurInterval surrogate_interval(const FieldArgs &f, double time) {
+  SurInterval v;
+  if (f.nt > 1) {
+    double tt, ta, tb;
+    int a0 = -1, a1 = -1;
+    if (!time_interval(f, time, a0, a1, tt, ta, tb)) {
+      v.err = (int)DEVERR_TIME_RANGE;
+      return v;
+    }
+    v.s0 = a0; v.s1 = a1;
+    v.tau = (float)((tt - ta) / (tb - ta));
+    if (f.period > 0.0) v.phase = (float)((tt - f.times[0]) / f.period);
+  }
+  return v;
+}
+
 // The 37 features of an alive particle (FP32 storage, interleaved U/V(/W)
-// slabs).  Returns 0, or a device error code (time outside the field, a
-// snapshot not resident) with o untouched.
+// slabs) whose time lies in iv.  Returns 0, or a device error code (time
+// outside the field, a snapshot not resident) with o untouched.
 __device__ __forceinline__ int surrogate_features(const GridArgs &g, const FieldArgs &f,
-                                                  float lon, float lat, float dep, double time,
-                                                  float (&o)[kSurFeat]) {
+                                                  float lon, float lat, float dep,
+                                                  const SurInterval &iv, float (&o)[kSurFeat]) {
+  if (iv.err) return iv.err;
   // cell and fractions
   const float q = wrap_lon(lon, g.lonf[0]);
   int i;
@@ -54,17 +77,8 @@ __device__ __forceinline__ int surrogate_features(const GridArgs &g, const Field
     k = axis_search<float>(g, 2, g.nz, z);
     zeta = __fdiv_rn(__fsub_rn(z, g.depthf[k]), __fsub_rn(g.depthf[k + 1], g.depthf[k]));
   }
-  // time interval
-  int s0 = 0, s1 = 0;
-  float tau = 0.f, phase = 0.f;
-  if (f.nt > 1) {
-    double tt, ta, tb;
-    int a0 = -1, a1 = -1;
-    if (!time_interval(f, time, a0, a1, tt, ta, tb)) return (int)DEVERR_TIME_RANGE;
-    s0 = a0; s1 = a1;
-    tau = (float)((tt - ta) / (tb - ta));
-    if (f.period > 0.0) phase = (float)((tt - f.times[0]) / f.period);
-  }
+  const int s0 = iv.s0, s1 = iv.s1;
+  const float tau = iv.tau, phase = iv.phase;
   const float *S0 = reinterpret_cast<const float *>(f.tab[s0]);
   const float *S1 = reinterpret_cast<const float *>(f.tab[s1]);
   if (!S0 || !S1) return (int)DEVERR_SLAB_MISSING;
