@@ -91,31 +91,54 @@ __device__ __forceinline__ float cos_deg(float lat) {
   return fmaf(x2, p, 1.0f);
 }
 
-// FP64 a / d, correctly rounded, for a divisor used many times, from r =
-// RN(1 / d): Markstein's correction (P. W. Markstein, IBM J. Res. Dev. 34(1),
-// 1990) -- q = a r, corrected once by its remainder, is within one unit in the
-// last place, and the second correction then rounds as the division does
-// (five instructions of the FP64 pipe, without a branch).  Dividends outside
-// 2^-639 .. 2^641 (zero, infinite and NaN ones among them) and divisors
-// whose reciprocal is marked unfit (0) are divided.
-__device__ __forceinline__ double reciprocal_for(double d) {
-  const unsigned e = ((unsigned)__double2hiint(d) >> 20) & 0x7ffu;
-  return e - 0x2ffu <= 0x200u ? 1.0 / d : 0.0;         // 2^-256 .. 2^257
-}
-__device__ __forceinline__ double quotient_refined(double a, double d, double r) {
-  double q = a * r;
-  q = fma(fma(-d, q, a), r, q);
-  return fma(fma(-d, q, a), r, q);
-}
+// FP64 a / d for a divisor used many times: a times the reciprocal held to
+// twice the precision, r + s with r = RN(1 / d) and s the rest, as RN(a r +
+// RN(a s)) (N. Brisebarre and J.-M. Muller, IEEE Trans. Comput. 57(2), 2008).
+// The sum is off by some 2^-106 before its one rounding, and no quotient of
+// two doubles lies much nearer than that to the middle between two others, so
+// it rounds as the division does: two instructions of the FP64 pipe and no
+// branch, for a dozen.  Dividends outside 2^-639 .. 2^641 (zero, infinite and
+// NaN ones among them) and divisors outside 2^-256 .. 2^257, whose reciprocal
+// is marked unfit (r = 0), are divided.
 __device__ __forceinline__ bool dividend_fit(double a) {
   return (((unsigned)__double2hiint(a) >> 20) & 0x7ffu) - 0x180u <= 0x500u;
 }
-__device__ __forceinline__ double quotient(double a, double d, double r) {
-  if (!dividend_fit(a) | (__double2hiint(r) == 0)) return a / d;
-  return quotient_refined(a, d, r);
+__device__ __forceinline__ void reciprocal_for(double d, double &r, double &s) {
+  const unsigned e = ((unsigned)__double2hiint(d) >> 20) & 0x7ffu;
+  const bool fit = e - 0x2ffu <= 0x200u;
+  r = fit ? 1.0 / d : 0.0;
+  s = fit ? fma(-d, r, 1.0) * r : 0.0;
 }
+__device__ __forceinline__ double times_reciprocal(double a, double r, double s) {
+  return fma(a, r, a * s);
+}
+__device__ __forceinline__ double quotient(double a, double d, double r, double s) {
+  return dividend_fit(a) & (__double2hiint(r) != 0) ? times_reciprocal(a, r, s) : a / d;
+}
+// A position's distance from its cell's lower face: fit as a dividend, or +0
+// (whose product is the +0 of the division).
+__device__ __forceinline__ bool fraction_fit(double a, double r) {
+  return (dividend_fit(a) | (__double_as_longlong(a) == 0)) & (__double2hiint(r) != 0);
+}
+// a / 6: 1/6 = r + s with s = (1 - 6 r) / 6, 6 r = 1 - 2^-54
 __device__ __forceinline__ double quotient6(double a) {
-  return dividend_fit(a) ? quotient_refined(a, 6.0, 1.0 / 6.0) : a / 6.0;
+  constexpr double r = 1.0 / 6.0, s = r / 18014398509481984.0;
+  return dividend_fit(a) ? times_reciprocal(a, r, s) : a / 6.0;
+}
+__device__ __forceinline__ bool is_nan_bits(double a) {
+  return ((unsigned long long)__double_as_longlong(a) << 1) > 0xffe0000000000000ull;
+}
+
+// FP64 order key: a < b exactly when key(a) < key(b), for finite a and b (both
+// zeros have one key); NaN lies outside every pair of finite keys.  Integer
+// comparisons, because the FP64 pipe is the bound: it takes 16 clocks of an
+// SM or more for each instruction of a warp, comparisons included.
+__device__ __forceinline__ long long order_key(double a) {
+  const long long b = __double_as_longlong(a);
+  return b < 0 ? (long long)0x8000000000000000ull - b : b;
+}
+__device__ __forceinline__ double from_order_key(long long k) {
+  return __longlong_as_double(k < 0 ? (long long)0x8000000000000000ull - k : k);
 }
 
 // u (m/s) -> degrees/s of longitude at latitude lat; v (m/s) -> degrees/s.
@@ -126,7 +149,7 @@ __device__ __forceinline__ float lon_rate(float u, float lat, const KernArgs &k)
   return __fdividef(u, k.deg_m_f * cos_deg(lat));
 }
 __device__ __forceinline__ double lat_rate(double v, const KernArgs &k) {
-  return dividend_fit(v) ? quotient_refined(v, k.deg_m, k.inv_deg_m) : v / k.deg_m;
+  return dividend_fit(v) ? times_reciprocal(v, k.inv_deg_m, k.inv_deg_m_rest) : v / k.deg_m;
 }
 __device__ __forceinline__ float lat_rate(float v, const KernArgs &k) { return v * k.inv_deg_m_f; }
 
@@ -179,15 +202,19 @@ struct Sampler {
   static constexpr int NC = D3 ? 8 : 4;
   // cached cell (ci = -1: none) and its bounds
   int ci, cj, ck;
-  Real xlo, xhi, ylo, yhi, zlo, zhi;
-  Real rx, ry, rz;            // 1 / (hi - lo)
-  Real dx, dy, dz;            // hi - lo, FP64 path only
+  Real xlo, xhi, ylo, yhi, zlo, zhi;   // FP32 path only
+  Real rx, ry, rz;            // 1 / (hi - lo); FP64: its leading part
+  // FP64 path only: the rest of the reciprocals, and the cell's bounds as
+  // order keys [klo, khi)
+  Real sx, sy, sz;
+  long long klo[3], khi[3];
   // cached snapshot interval and the snapshots whose corners are held
   int s0;                     // first snapshot of the cached pair (second: snap_next)
   // what `v` lacks: 1 the cell changed, 2 the snapshot pair moved on by one
   // (s0 is the old s1), 4 anything else (a new pair, or nothing held yet)
   int dirty;
-  double ta;                  // FP32 path: interval start in unwrapped time
+  double ta;                  // FP32 path: interval start in unwrapped time;
+  double tb, rt, st;          // FP64 path: the interval and the reciprocal of its length
   float span, rspan;          // FP32 path
   // Corner values.  PAIRS (FP32): (U, V) of a corner as one pair -- the layout
   // they are loaded in, and the operand of packed multiply-adds -- and W of
@@ -231,6 +258,10 @@ struct Sampler {
     xlo = (Real)1; xhi = (Real)0;
     ylo = (Real)1; yhi = (Real)0;
     zlo = (Real)1; zhi = (Real)0;
+    if constexpr (sizeof(Real) == 8) {
+      for (int a = 0; a < 3; ++a) { klo[a] = 1; khi[a] = 0; }
+      ta = tb = rt = st = 0.0;
+    }
   }
 };
 
@@ -257,14 +288,6 @@ __device__ __forceinline__ float wrap_lon(float p, float x0) {
     q = x0 + r;
   }
   return q;
-}
-
-// Is p inside the cached cell [lo, hi]?  FP64: the definition's half-open
-// cell, closed only at the last node.  FP32: closed on both sides.
-template <typename Real>
-__device__ __forceinline__ bool in_cell(Real p, Real lo, Real hi, bool last) {
-  if constexpr (sizeof(Real) == 8) return p >= lo && (p < hi || (last && p == hi));
-  else return p >= lo && p <= hi;
 }
 
 // Snapshot interval for time t in FP64 (the definition's rules: the largest
@@ -605,7 +628,12 @@ __device__ __forceinline__ int sample_fields(const A &a, Sampler<Real, Store, NF
       }
       if (s0 != c.s0) c.dirty |= (c.s0 >= 0 && s0 == snap_next(a.f, c.s0)) ? 2 : 4;
       c.s0 = s0;
-      tau = (tt - ta) / (tb - ta);
+      if (__double_as_longlong(ta) != __double_as_longlong(c.ta) ||
+          __double_as_longlong(tb) != __double_as_longlong(c.tb)) {
+        c.ta = ta; c.tb = tb;
+        reciprocal_for(tb - ta, c.rt, c.st);
+      }
+      tau = quotient(tt - ta, tb - ta, c.rt, c.st);
     } else {
       c.s0 = 0;
     }
@@ -623,7 +651,7 @@ __device__ __forceinline__ int sample_fields(const A &a, Sampler<Real, Store, NF
                                    : interp_space<Real, NC>(c.v[1][f], xi, eta, zeta);
         val = val + (b - val) * tau;
       }
-      if (!(val == val)) return 3;
+      if (is_nan_bits(val)) return 3;
       vel[f] = val;
     }
     if constexpr (NF == 2) vel[2] = (Real)0;

@@ -26,53 +26,42 @@
 
 namespace pg {
 
-// FP64: locate p on the longitude axis, using and refreshing the cache.
-// Returns false when the position is out of the domain.  The cached cell is
-// tested first: a position inside it is inside the domain.  (The FP64 pipe
-// takes a warp instruction every 16 clocks of an SM, comparisons included, so
-// the stage's time is its count of FP64 instructions.)
-template <typename Real, typename Store, int NF, bool D3, int GEO>
-__device__ __forceinline__ bool locate_lon(const GridArgs &g, Sampler<Real, Store, NF, D3, GEO> &c,
-                                           Real p, Real &xi) {
-  Real q = p;
-  const Real *x = axis<Real>(g, 0);
-  if (is_per<GEO>(g)) {
-    if (!isfinite(p)) return false;
-    q = wrap_lon(p, axis_lo(g, 0, p));
-  }
-  if (!(c.ci >= 0 && in_cell<Real>(q, c.xlo, c.xhi, c.ci == g.nx - 2 && !is_per<GEO>(g)))) {
-    if (!is_per<GEO>(g) && !(p >= axis_lo(g, 0, p) && p <= axis_hi(g, 0, p))) return false;
-    c.dirty |= 1;
-    if (is_per<GEO>(g) && q >= axis_hi(g, 0, p)) {
-      c.ci = g.nx - 1;
-      c.xlo = x[g.nx - 1];
-      c.xhi = lon_end(g, p);
-    } else {
-      const int i = axis_search<Real>(g, 0, g.nx, q);
-      c.ci = i;
-      c.xlo = x[i]; c.xhi = x[i + 1];
-    }
-    c.dx = c.xhi - c.xlo;
-    c.rx = reciprocal_for(c.dx);
-  }
-  xi = quotient(q - c.xlo, c.dx, c.rx);
-  return true;
+// FP64 slow path: locate p, known to lie outside the cached cell of index ci
+// on axis a (n nodes; the last cell is closed when CLOSED): the neighbour
+// where it holds p, else a search.  Refreshes the cell: its index, the
+// reciprocal of its width, and its bounds as order keys.  Returns
+// false when p is outside the axis.  The cell found is the largest i <= n-2
+// with x[i] <= p.
+__device__ __forceinline__ void set_cell64(double lo, double hi, bool closed, double &r, double &s,
+                                           long long &klo, long long &khi) {
+  reciprocal_for(hi - lo, r, s);
+  klo = order_key(lo);
+  khi = order_key(hi) + (closed ? 1 : 0);
 }
-
-template <typename Real>
-__device__ __forceinline__ bool locate_axis(const GridArgs &g, int a, int n, int &ci, Real &lo,
-                                            Real &hi, Real &d, Real &rinv, Real p, Real &xi,
-                                            int &dirty) {
-  const Real *x = axis<Real>(g, a);
-  if (!(ci >= 0 && in_cell<Real>(p, lo, hi, ci == n - 2))) {
-    if (!(p >= x[0] && p <= x[n - 1])) return false;
-    const int i = axis_search<Real>(g, a, n, p);
-    ci = i; lo = x[i]; hi = x[i + 1];
-    dirty |= 1;
-    d = hi - lo;
-    rinv = reciprocal_for(d);
+template <bool CLOSED>
+__device__ __forceinline__ bool relocate64(const GridArgs &g, int a, int n, double p, int &ci,
+                                           double &r, double &s, long long &klo, long long &khi) {
+  const double *x = axis<double>(g, a);
+  int i = -1;
+  double lo = 0.0, hi = 0.0;
+  if (ci >= 0 && ci <= n - 2) {
+    if (order_key(p) < klo) {
+      if (ci >= 1) {
+        lo = x[ci - 1]; hi = x[ci];
+        if (lo <= p) i = ci - 1;
+      }
+    } else if (ci + 1 <= n - 2) {
+      lo = x[ci + 1]; hi = x[ci + 2];
+      if (p < hi || (CLOSED && ci + 1 == n - 2 && p == hi)) i = ci + 1;
+    }
   }
-  xi = quotient(p - lo, d, rinv);
+  if (i < 0) {
+    if (!(p >= x[0] && p <= x[n - 1])) return false;
+    i = axis_search<double>(g, a, n, p);
+    lo = x[i]; hi = x[i + 1];
+  }
+  ci = i;
+  set_cell64(lo, hi, CLOSED && i == n - 2, r, s, klo, khi);
   return true;
 }
 
@@ -227,21 +216,71 @@ __device__ __forceinline__ int velocity(const A &a, Sampler<Real, Store, NF, D3,
     }
     return 0;
   }
-  Real xi, eta, zeta = (Real)0;
-  if (!locate_lon(g, c, lon, xi)) return 1;
-  if (!locate_axis<Real>(g, 1, g.ny, c.cj, c.ylo, c.yhi, c.dy, c.ry, lat, eta, c.dirty)) return 1;
-  if constexpr (D3) {
-    if (!locate_axis<Real>(g, 2, g.nz, c.ck, c.zlo, c.zhi, c.dz, c.rz, dep, zeta, c.dirty)) return 2;
-  } else {
-    c.ck = 0;
+  if constexpr (sizeof(Real) == 8) {
+    // FP64: as in FP32, one predicate over the cached cell on every axis --
+    // half-open, closed at an axis' last node: the bounds are kept as order
+    // keys [lo, hi) with hi one up where the cell is closed -- so that the
+    // common stage is one block in which the axes' chains overlap.
+    double q = lon;
+    if (is_per<GEO>(g)) {
+      if (!isfinite(lon)) return 1;
+      q = wrap_lon(lon, axis_lo(g, 0, lon));
+    }
+    const long long kx = order_key(q), ky = order_key(lat);
+    bool hx = (kx >= c.klo[0]) & (kx < c.khi[0]);
+    const bool hy = (ky >= c.klo[1]) & (ky < c.khi[1]);
+    bool hz = true;
+    if constexpr (D3) {
+      const long long kz = order_key(dep);
+      hz = (kz >= c.klo[2]) & (kz < c.khi[2]);
+    }
+    if (!(hx & hy & hz)) {
+      if (!hx) {
+        if (is_per<GEO>(g)) {
+          if (q >= axis_hi(g, 0, q)) {          // the wrap cell
+            c.ci = g.nx - 1;
+            set_cell64(axis_hi(g, 0, q), lon_end(g, q), false, c.rx, c.sx, c.klo[0], c.khi[0]);
+          } else if (!relocate64<false>(g, 0, g.nx, q, c.ci, c.rx, c.sx, c.klo[0], c.khi[0])) {
+            return 1;
+          }
+        } else if (!relocate64<true>(g, 0, g.nx, q, c.ci, c.rx, c.sx, c.klo[0], c.khi[0])) {
+          return 1;
+        }
+        c.dirty |= 1;
+      }
+      if (!hy) {
+        if (!relocate64<true>(g, 1, g.ny, lat, c.cj, c.ry, c.sy, c.klo[1], c.khi[1])) return 1;
+        c.dirty |= 1;
+      }
+      if constexpr (D3) {
+        if (!hz) {
+          if (!relocate64<true>(g, 2, g.nz, dep, c.ck, c.rz, c.sz, c.klo[2], c.khi[2])) return 2;
+          c.dirty |= 1;
+        }
+      } else {
+        c.ck = 0;
+      }
+    }
+    const double xlo = from_order_key(c.klo[0]), ylo = from_order_key(c.klo[1]);
+    const double zlo = D3 ? from_order_key(c.klo[2]) : 0.0;
+    const double ax = q - xlo, ay = lat - ylo, az = D3 ? dep - zlo : 0.0;
+    double xi = times_reciprocal(ax, c.rx, c.sx), eta = times_reciprocal(ay, c.ry, c.sy);
+    double zeta = D3 ? times_reciprocal(az, c.rz, c.sz) : 0.0;
+    bool fit = fraction_fit(ax, c.rx) & fraction_fit(ay, c.ry);
+    if constexpr (D3) fit = fit & fraction_fit(az, c.rz);
+    if (!fit) {
+      xi = ax / ((c.ci == g.nx - 1 ? lon_end(g, q) : g.lon[c.ci + 1]) - g.lon[c.ci]);
+      eta = ay / (g.lat[c.cj + 1] - g.lat[c.cj]);
+      if constexpr (D3) zeta = az / (g.depth[c.ck + 1] - g.depth[c.ck]);
+    }
+    const int r = sample_fields(a, c, ck, off, xi, eta, zeta, vel);
+    if (r) return r;
+    if (is_sph<GEO>(g)) {
+      vel[0] = lon_rate(vel[0], lat, a.k);
+      vel[1] = lat_rate(vel[1], a.k);
+    }
+    return 0;
   }
-  const int r = sample_fields(a, c, ck, off, xi, eta, zeta, vel);
-  if (r) return r;
-  if (is_sph<GEO>(g)) {
-    vel[0] = lon_rate(vel[0], lat, a.k);
-    vel[1] = lat_rate(vel[1], a.k);
-  }
-  return 0;
 }
 
 // Parameters of the worked example's behaviours per Real.

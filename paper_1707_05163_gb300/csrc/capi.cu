@@ -504,6 +504,7 @@ pg_status resolve_kernel(const pg_kernel *k, const pg_fieldset *fs, uint64_t see
     return PG_ERR_ARG;
   }
   a.seed = seed; a.deg_m = 1852.0 * 60.0; a.inv_deg_m = 1.0 / a.deg_m;
+  a.inv_deg_m_rest = std::fma(-a.deg_m, a.inv_deg_m, 1.0) * a.inv_deg_m;
   a.deg_m_f = (float)a.deg_m; a.inv_deg_m_f = (float)(1.0 / a.deg_m);
   a.kh_f = (float)a.kh; a.w_sink_f = (float)a.w_sink;
   a.dwell_f = (float)a.dwell;

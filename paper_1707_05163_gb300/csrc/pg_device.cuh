@@ -57,7 +57,7 @@ struct KernArgs {
   double kh, w_sink;
   uint64_t seed;
   double deg_m;              // metres per degree
-  double inv_deg_m;          // RN(1 / deg_m)
+  double inv_deg_m, inv_deg_m_rest;   // 1 / deg_m in two parts
   float deg_m_f, inv_deg_m_f, kh_f, w_sink_f;   // FP32 copies for the FP32 path
   double dwell = 0.0, max_age = 0.0;   // settle: dwelling depth (m); age: deletion age (s)
   float dwell_f = 0.f;
