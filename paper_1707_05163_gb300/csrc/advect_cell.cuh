@@ -41,6 +41,19 @@ __device__ __forceinline__ bool norm_axis(int &i, float &f, int n, bool periodic
   return false;
 }
 
+// norm_axis for an offset at most one cell away and an index that stays
+// inside -- the common move, without a branch; ok is cleared for anything
+// else (a whole-cell remainder of 1, NaN, the last node, the outside), whose
+// index and offset are then those of norm_axis from the start.
+__device__ __forceinline__ void shift_axis(int &i, float &f, int n, bool periodic, bool &ok) {
+  const bool dn = f < 0.f, up = f >= 1.f;
+  f = dn ? f + 1.0f : (up ? f - 1.0f : f);
+  i += (up ? 1 : 0) - (dn ? 1 : 0);
+  ok = ok & (f >= 0.f) & (f < 1.f);
+  if (periodic) i = i < 0 ? i + n : (i >= n ? i - n : i);
+  else ok = ok & ((unsigned)i <= (unsigned)(n - 2));
+}
+
 // Velocity in cells per second at the stage position base + kc * off.
 template <typename Store, int NF, bool D3, int GEO>
 __device__ __forceinline__ int velocity_cell(const StepArgs &a, Sampler<float, Store, NF, D3, GEO> &c,
@@ -52,11 +65,19 @@ __device__ __forceinline__ int velocity_cell(const StepArgs &a, Sampler<float, S
   // No NaN test on the stage velocity: a NaN velocity makes the next stage
   // offset (or the step's result) NaN, which fails normalisation, and a
   // failure on a NaN offset reports PG_NAN, with the state kept.
-  const int nan = (!(x == x) | !(y == y) | !(z == z)) ? 3 : 0;
-  if (!norm_axis(i, x, g.nx, is_per<GEO>(g))) return nan ? nan : 1;
-  if (!norm_axis(j, y, g.ny, false)) return nan ? nan : 1;
-  if constexpr (D3) {
-    if (!norm_axis(k, z, g.nz, false)) return nan ? nan : 2;
+  const float x0 = x, y0 = y, z0 = z;
+  bool ok = true;
+  shift_axis(i, x, g.nx, is_per<GEO>(g), ok);
+  shift_axis(j, y, g.ny, false, ok);
+  if constexpr (D3) shift_axis(k, z, g.nz, false, ok);
+  if (!ok) {
+    i = b.i; j = b.j; k = b.k; x = x0; y = y0; z = z0;
+    const int nan = (!(x == x) | !(y == y) | !(z == z)) ? 3 : 0;
+    if (!norm_axis(i, x, g.nx, is_per<GEO>(g))) return nan ? nan : 1;
+    if (!norm_axis(j, y, g.ny, false)) return nan ? nan : 1;
+    if constexpr (D3) {
+      if (!norm_axis(k, z, g.nz, false)) return nan ? nan : 2;
+    }
   }
   if (i != c.ci || j != c.cj || (D3 && k != c.ck)) {
     c.ci = i;

@@ -34,17 +34,20 @@ __device__ __forceinline__ void load_node(const float *p, size_t node, const flo
   }
 }
 
-// Quantised storage: value = float(code) * scale, rounded in FP32.
+// Quantised storage: value = float(code) * scale, rounded in FP32 (two to an
+// instruction).
 template <typename Real, int NF>
 __device__ __forceinline__ void load_node(const __half *p, size_t node, const float *sc, Real (&v)[NF]) {
   if constexpr (NF == 2) {
     const __half2 a = __ldg(reinterpret_cast<const __half2 *>(p) + node);
-    v[0] = (Real)(__low2float(a) * sc[0]); v[1] = (Real)(__high2float(a) * sc[1]);
+    const float2 b = __fmul2_rn(make_float2(__low2float(a), __high2float(a)), make_float2(sc[0], sc[1]));
+    v[0] = (Real)b.x; v[1] = (Real)b.y;
   } else {
     const uint2 a = __ldg(reinterpret_cast<const uint2 *>(p) + node);
     const __half2 lo = *reinterpret_cast<const __half2 *>(&a.x);
     const __half2 hi = *reinterpret_cast<const __half2 *>(&a.y);
-    v[0] = (Real)(__low2float(lo) * sc[0]); v[1] = (Real)(__high2float(lo) * sc[1]);
+    const float2 b = __fmul2_rn(make_float2(__low2float(lo), __high2float(lo)), make_float2(sc[0], sc[1]));
+    v[0] = (Real)b.x; v[1] = (Real)b.y;
     v[2] = (Real)(__low2float(hi) * sc[2]);
   }
 }
@@ -53,12 +56,14 @@ template <typename Real, int NF>
 __device__ __forceinline__ void load_node(const __nv_bfloat16 *p, size_t node, const float *sc, Real (&v)[NF]) {
   if constexpr (NF == 2) {
     const __nv_bfloat162 a = __ldg(reinterpret_cast<const __nv_bfloat162 *>(p) + node);
-    v[0] = (Real)(__low2float(a) * sc[0]); v[1] = (Real)(__high2float(a) * sc[1]);
+    const float2 b = __fmul2_rn(make_float2(__low2float(a), __high2float(a)), make_float2(sc[0], sc[1]));
+    v[0] = (Real)b.x; v[1] = (Real)b.y;
   } else {
     const uint2 a = __ldg(reinterpret_cast<const uint2 *>(p) + node);
     const __nv_bfloat162 lo = *reinterpret_cast<const __nv_bfloat162 *>(&a.x);
     const __nv_bfloat162 hi = *reinterpret_cast<const __nv_bfloat162 *>(&a.y);
-    v[0] = (Real)(__low2float(lo) * sc[0]); v[1] = (Real)(__high2float(lo) * sc[1]);
+    const float2 b = __fmul2_rn(make_float2(__low2float(lo), __high2float(lo)), make_float2(sc[0], sc[1]));
+    v[0] = (Real)b.x; v[1] = (Real)b.y;
     v[2] = (Real)(__low2float(hi) * sc[2]);
   }
 }
@@ -334,38 +339,63 @@ __device__ __forceinline__ int snap_next(const FieldArgs &f, int s0) {
   return s0 + 1 < f.nt ? s0 + 1 : 0;
 }
 
+// Byte offsets of the cached cell's corners in a slab: the first corner, and
+// the steps to its neighbours in longitude (the periodic wrap cell joins node
+// nx-1 to node 0), latitude and depth.
+struct CornerOffsets {
+  size_t first, dy, dz;
+  ptrdiff_t dx;
+};
+
+// false: the cached cell is no cell of the grid (the wrap cell is nx-1) -- an
+// internal error recorded in a.err, never a read outside the slab.
+template <typename Real, typename Store, int NF, bool D3, int GEO, class A>
+__device__ __forceinline__ bool corner_offsets(const A &a, const Sampler<Real, Store, NF, D3, GEO> &c,
+                                               CornerOffsets &o) {
+  constexpr int EB = (NF == 2 ? 2 : 4) * (int)sizeof(Store);
+  const GridArgs &g = a.g;
+  if (!(((unsigned)c.ci < (unsigned)g.nx) & ((unsigned)c.cj <= (unsigned)(g.ny - 2)) &
+        (D3 ? (unsigned)c.ck <= (unsigned)(g.nz - 2) : c.ck == 0))) {
+    atomicCAS(a.err, 0, (int)DEVERR_CELL_INDEX);
+    return false;
+  }
+  const unsigned row = (D3 ? (unsigned)c.ck * (unsigned)g.ny : 0u) + (unsigned)c.cj;
+  o.first = ((size_t)row * (unsigned)g.nx + (unsigned)c.ci) * EB;
+  o.dx = (ptrdiff_t)((c.ci + 1 == g.nx ? 1 - g.nx : 1) * EB);
+  o.dy = (size_t)(unsigned)g.nx * EB;
+  o.dz = o.dy * (unsigned)g.ny;
+  return true;
+}
+
+// The corners in snapshot s into slot sl.
 template <typename Real, typename Store, int NF, bool D3, int GEO, class A>
 __device__ __forceinline__ bool gather_slab(const A &a, Sampler<Real, Store, NF, D3, GEO> &c,
-                                            int sl, int s) {
-  const GridArgs &g = a.g;
-  const Store *base = reinterpret_cast<const Store *>(a.f.tab[s]);
+                                            const CornerOffsets &o, int sl, int s) {
+  const char *base = reinterpret_cast<const char *>(a.f.tab[s]);
   if (base == nullptr) {
     atomicCAS(a.err, 0, (int)DEVERR_SLAB_MISSING);
     return false;
   }
-  // the cached cell must be a cell of the grid (the periodic wrap cell is
-  // nx-1, joining node nx-1 to node 0); anything else is an internal error
-  // recorded in a.err, never a read outside the slab
-  if (!((unsigned)c.ci < (unsigned)g.nx && (unsigned)c.cj <= (unsigned)(g.ny - 2) &&
-        (!D3 || (unsigned)c.ck <= (unsigned)(g.nz - 2)) && (D3 || c.ck == 0))) {
-    atomicCAS(a.err, 0, (int)DEVERR_CELL_INDEX);
-    return false;
-  }
-  const int ci1 = c.ci + 1 == g.nx ? 0 : c.ci + 1;   // the periodic wrap cell joins nx-1 to 0
   float sc[3] = {1.f, 1.f, 1.f};
-  if (a.f.scales != nullptr) {
+  if constexpr (sizeof(Store) == 2) {
+    if constexpr (NF == 2) {
+      const float2 v = reinterpret_cast<const float2 *>(a.f.scales)[s];
+      sc[0] = v.x; sc[1] = v.y;
+    } else {
 #pragma unroll
-    for (int f = 0; f < NF; ++f) sc[f] = a.f.scales[s * NF + f];
+      for (int f = 0; f < NF; ++f) sc[f] = a.f.scales[s * NF + f];
+    }
   }
+  base += o.first;
 #pragma unroll
   for (int kk = 0; kk < (D3 ? 2 : 1); ++kk) {
 #pragma unroll
     for (int jj = 0; jj < 2; ++jj) {
-      const size_t row = ((size_t)(c.ck + kk) * g.ny + (size_t)(c.cj + jj)) * g.nx;
 #pragma unroll
       for (int ii = 0; ii < 2; ++ii) {
+        const char *p = base + (kk ? o.dz : 0) + (jj ? o.dy : 0) + (ii ? o.dx : 0);
         Real vv[NF];
-        load_node<Real, NF>(base, row + (size_t)(ii ? ci1 : c.ci), sc, vv);
+        load_node<Real, NF>(reinterpret_cast<const Store *>(p), 0, sc, vv);
         c.put(sl, kk * 4 + jj * 2 + ii, vv);
       }
     }
@@ -379,15 +409,17 @@ __device__ __forceinline__ bool gather_slab(const A &a, Sampler<Real, Store, NF,
 template <typename Real, typename Store, int NF, bool D3, int GEO, class A>
 __device__ __forceinline__ bool gather(const A &a, Sampler<Real, Store, NF, D3, GEO> &c,
                                        bool steady) {
+  CornerOffsets o;
+  if (!corner_offsets(a, c, o)) return false;
   if (steady) {
-    if (!gather_slab(a, c, 0, c.s0)) return false;
+    if (!gather_slab(a, c, o, 0, c.s0)) return false;
     if constexpr (sizeof(Real) == 4) c.template move<0>();     // FP32 interpolates both slots
   } else if (c.dirty == 2) {
     c.template move<1>();
-    if (!gather_slab(a, c, 1, snap_next(a.f, c.s0))) return false;
+    if (!gather_slab(a, c, o, 1, snap_next(a.f, c.s0))) return false;
   } else {
-    if (!gather_slab(a, c, 0, c.s0)) return false;
-    if (!gather_slab(a, c, 1, snap_next(a.f, c.s0))) return false;
+    if (!gather_slab(a, c, o, 0, c.s0)) return false;
+    if (!gather_slab(a, c, o, 1, snap_next(a.f, c.s0))) return false;
   }
   c.dirty = 0;
   return true;
