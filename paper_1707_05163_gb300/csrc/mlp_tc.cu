@@ -81,8 +81,22 @@ __host__ __device__ constexpr uint32_t instr_desc(int m, int n) {
          ((uint32_t)(m >> 4) << 24);
 }
 
-// 16 FP32 values rounded to BF16 (nearest even, in pairs) and written as two
-// 16-byte stores; dst must be 16-byte aligned.
+// 32 bytes in one store or load (dst, src 32-byte aligned): a lane of these
+// kernels has a row's columns to itself, so 16-byte accesses touch every
+// 32-byte sector of the row twice.
+__device__ __forceinline__ void store32(void *dst, const uint32_t (&w)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n" ::"l"(dst), "r"(w[0]),
+               "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+               : "memory");
+}
+__device__ __forceinline__ void load32(const void *src, uint32_t (&w)[8]) {
+  asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+               : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]),
+                 "=r"(w[6]), "=r"(w[7])
+               : "l"(src));
+}
+
+// 16 FP32 values rounded to BF16 (nearest even, in pairs), one 32-byte store.
 __device__ __forceinline__ void store_bf16x16(__nv_bfloat16 *dst, const float (&v)[16]) {
   uint32_t w[8];
 #pragma unroll
@@ -90,8 +104,18 @@ __device__ __forceinline__ void store_bf16x16(__nv_bfloat16 *dst, const float (&
     const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
     w[j] = *reinterpret_cast<const uint32_t *>(&h);
   }
-  reinterpret_cast<uint4 *>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
-  reinterpret_cast<uint4 *>(dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+  store32(dst, w);
+}
+
+// 16 FP32 values in two 32-byte stores.
+__device__ __forceinline__ void store_f32x16(float *dst, const float (&v)[16]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t w[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) w[j] = __float_as_uint(v[8 * h + j]);
+    store32(dst + 8 * h, w);
+  }
 }
 
 // Sums over the warp's 32 lanes of 16 values per lane: a reduce-scatter of 16
@@ -252,8 +276,7 @@ gemm_tc_kernel(const __nv_bfloat16 *__restrict__ A, int lda, const __nv_bfloat16
 #pragma unroll
       for (int j = 0; j < 16; ++j) v[j] = row < M ? __uint_as_float(r[j]) : 0.f;
       if (row < M) {
-        // 16 consecutive columns of this thread's row: 16-byte vector loads
-        // of the bias and 16-byte stores (32 B of BF16 or 64 B of FP32)
+        // 16 consecutive columns of this thread's row
         const size_t o = (size_t)row * ldc + c0;
         if (bias) {
 #pragma unroll
@@ -267,10 +290,9 @@ gemm_tc_kernel(const __nv_bfloat16 *__restrict__ A, int lda, const __nv_bfloat16
 #pragma unroll
           for (int j = 0; j < 16; ++j) v[j] = gelu_tc(v[j]);
         } else if (act == 2) {
-          // times GELU'(g): 16 BF16 pre-activations in two 16-byte loads
-          const uint4 g0 = *reinterpret_cast<const uint4 *>(gin + o);
-          const uint4 g1 = *reinterpret_cast<const uint4 *>(gin + o + 8);
-          const uint32_t gw[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+          // times GELU'(g): 16 BF16 pre-activations in one load
+          uint32_t gw[8];
+          load32(gin + o, gw);
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162 *>(&gw[j]);
@@ -278,11 +300,7 @@ gemm_tc_kernel(const __nv_bfloat16 *__restrict__ A, int lda, const __nv_bfloat16
             v[2 * j + 1] *= gelu_grad_tc(__high2float(h));
           }
         }
-        if (out_f32) {
-#pragma unroll
-          for (int j = 0; j < 16; j += 4)
-            *reinterpret_cast<float4 *>(out_f32 + o + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-        }
+        if (out_f32) store_f32x16(out_f32 + o, v);
         if (out_bf16) store_bf16x16(out_bf16 + o, v);
       }
       if (colpart) {
@@ -342,7 +360,8 @@ int gemm_tc_max_ctas() {
 }
 
 // Products of the MLP on tcgen05; N and K must be 64 or 256, all row
-// strides multiples of 8 elements, bias and outputs 16-byte aligned.
+// strides multiples of 8 elements (ldc of 16), bias 16-byte and outputs 32-byte
+// aligned.
 // colpart (may be null): column sums of the result over each CTA's rows,
 // [*nparts][N] FP32, from the values before they are rounded to BF16.  *err
 // (device) is set to 1 if a CTA gave up waiting for its accumulator.
@@ -351,9 +370,9 @@ cudaError_t gemm_nt_tc(const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, 
                        __nv_bfloat16 *out_bf16, __nv_bfloat16 *pre_bf16, int ldc, cudaStream_t st,
                        int *err, const __nv_bfloat16 *gin, float *colpart, int *nparts) {
   if (M == 0) return cudaSuccess;
-  if (lda % 8 || ldb % 8 || ldc % 8 || !err || (act == 2 && !gin)) return cudaErrorInvalidValue;
-  if (((uintptr_t)bias | (uintptr_t)out_f32 | (uintptr_t)out_bf16 | (uintptr_t)pre_bf16 |
-       (uintptr_t)gin) % 16)
+  if (lda % 8 || ldb % 8 || ldc % 16 || !err || (act == 2 && !gin)) return cudaErrorInvalidValue;
+  if ((uintptr_t)bias % 16 || ((uintptr_t)out_f32 | (uintptr_t)out_bf16 | (uintptr_t)pre_bf16 |
+                               (uintptr_t)gin) % 32)
     return cudaErrorInvalidValue;
   if (N == 256 && K == 256)
     return launch_tc<256, 256>(A, lda, B, ldb, M, bias, act, out_f32, out_bf16, pre_bf16, gin, ldc, colpart, nparts, st, err);
@@ -518,11 +537,10 @@ gemm_splitk_tc_kernel(const __nv_bfloat16 *__restrict__ A, int64_t lda, int Mrow
             "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
           : "r"(taddr));
       asm volatile("tcgen05.wait::ld.sync.aligned;\n");
+      float v[16];
 #pragma unroll
-      for (int j = 0; j < 16; j += 4)
-        *reinterpret_cast<float4 *>(out + cc + j) =
-            make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]),
-                        __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
+      for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+      store_f32x16(out + cc, v);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n");
@@ -609,7 +627,7 @@ cudaError_t gemm_tn_splitk_tc(const __nv_bfloat16 *A, int64_t lda, int Mrows,
                               float *scratch, size_t scratch_bytes, const float *bpart, int nparts,
                               float *bout, cudaStream_t st, int *err) {
   if (K == 0 || Mrows == 0) return cudaSuccess;
-  if (lda % 8 || ldb % 8 || !err || (Mrows != 64 && Mrows != 256) || ((uintptr_t)scratch % 16) ||
+  if (lda % 8 || ldb % 8 || !err || (Mrows != 64 && Mrows != 256) || ((uintptr_t)scratch % 32) ||
       !bpart || !bout)
     return cudaErrorInvalidValue;
   if (((uintptr_t)A | (uintptr_t)B) % 16) return cudaErrorInvalidValue;
