@@ -298,8 +298,8 @@ __global__ void pack_input(const float *x, int64_t M, int n_real, int ld, __nv_b
 
 // MSE loss 0.5 * mean over rows of sum over the n_out outputs of (y - t)^2
 // with output gradient (y - t) / M in FP32 and BF16 (padded columns zero),
-// eight columns per thread (ldy a multiple of 64).
-__global__ void mse_grad(const float *y, int ldy, const float *t, int n_out, int64_t M,
+// eight columns per thread (ldy a multiple of 64; y has row stride ys).
+__global__ void mse_grad(const float *y, int ys, int ldy, const float *t, int n_out, int64_t M,
                          float *dy, __nv_bfloat16 *dyb, float *loss_partial) {
   __shared__ float sh[256];
   const int cpr = ldy / 8;
@@ -314,7 +314,7 @@ __global__ void mse_grad(const float *y, int ldy, const float *t, int n_out, int
     for (int j = 0; j < 8; ++j) {
       g[j] = 0.f;
       if (c0 + j < n_out) {
-        const float d = y[r * ldy + c0 + j] - t[r * n_out + c0 + j];
+        const float d = y[r * ys + c0 + j] - t[r * n_out + c0 + j];
         l += 0.5f * d * d;
         g[j] = d / (float)M;
       }
@@ -409,11 +409,10 @@ struct pg_mlp {
   float *y = nullptr;                 // output [cap x pout] FP32
   float *dy = nullptr;                // FP32 gradient of the current layer output [cap x width]
   __nv_bfloat16 *dyb = nullptr, *dyt = nullptr, *xt = nullptr;   // BF16 grads, transposes
-  __nv_bfloat16 *dyb2 = nullptr;      // second BF16 gradient buffer (tcgen05 input gradient)
   float *gscratch = nullptr;          // split-K partials of the weight gradient
   size_t gscratch_bytes = 0;
   float *loss_partial = nullptr;
-  float *colpart = nullptr;           // column-sum partials of the bias gradients
+  float *colpart = nullptr;           // column-sum partials of the bias gradients, per layer
   int col_rows = 0;                   // its rows: at most this many partials
   int use_tc = 0;                     // tcgen05 products when available
   int fused = 1;                      // tcgen05 inference in one fused kernel when the shape allows
@@ -433,14 +432,13 @@ size_t mlp_fused_packed_bytes();
 cudaError_t mlp_fused_pack(const __nv_bfloat16 *const w[5], uint8_t *out, cudaStream_t st);
 cudaError_t mlp_fused_forward(const float *x, int64_t M, int n_in, const uint8_t *wpk,
                               const float *const bias[5], float *y, int n_out, cudaStream_t st,
-                              int *err);
+                              int *err, __nv_bfloat16 *const *pre = nullptr,
+                              __nv_bfloat16 *const *act = nullptr);
 cudaError_t mlp_fused_step_launch(const SurrogateStepIO &io, uint8_t *xpk, const uint8_t *wpk,
                                   const float *const bias[5], cudaStream_t st, int *err);
 cudaError_t mlp_wait_probe(long long polls, int *err, cudaStream_t st);
-cudaError_t gemm_tn_splitk_tc(const __nv_bfloat16 *A, int64_t lda, int Mrows,
-                              const __nv_bfloat16 *B, int64_t ldb, int N, int64_t K, float *out,
-                              float *scratch, size_t scratch_bytes, const float *bpart, int nparts,
-                              float *bout, cudaStream_t st, int *err);
+cudaError_t gemm_tn_splitk_tc(const WeightGrad *w, int ng, int64_t K, float *scratch,
+                              size_t scratch_bytes, cudaStream_t st, int *err);
 }
 
 namespace {
@@ -452,8 +450,8 @@ void free_ws(pg_mlp *n) {
   n->act.clear();
   n->pre.clear();
   dev_free(n->y); dev_free(n->dy); dev_free(n->dyb); dev_free(n->dyt); dev_free(n->xt);
-  dev_free(n->dyb2); dev_free(n->gscratch);
-  n->dyb2 = nullptr; n->gscratch = nullptr; n->gscratch_bytes = 0;
+  dev_free(n->gscratch);
+  n->gscratch = nullptr; n->gscratch_bytes = 0;
   dev_free(n->loss_partial); dev_free(n->colpart);
   n->colpart = nullptr;
   n->x0 = nullptr; n->y = nullptr; n->dy = nullptr; n->dyb = nullptr; n->dyt = nullptr;
@@ -481,7 +479,6 @@ cudaError_t ensure_ws(pg_mlp *n, int64_t rows) {
   al((void **)&n->y, cap * n->pout * 4);
   al((void **)&n->dy, cap * wmax * 4);
   al((void **)&n->dyb, cap * wmax * 2);
-  al((void **)&n->dyb2, cap * wmax * 2);
   // split-K partials: up to 64 splits of a 256 x 256 product
   n->gscratch_bytes = (size_t)64 * 256 * 256 * sizeof(float);
   al((void **)&n->gscratch, n->gscratch_bytes);
@@ -489,7 +486,7 @@ cudaError_t ensure_ws(pg_mlp *n, int64_t rows) {
   al((void **)&n->xt, cap * std::max(n->width, n->pin) * 2);
   al((void **)&n->loss_partial, 1024 * 4);
   n->col_rows = std::max(gemm_tc_max_ctas(), 128);
-  al((void **)&n->colpart, (size_t)n->col_rows * wmax * 4);
+  al((void **)&n->colpart, (size_t)n->nl * n->col_rows * wmax * 4);
   if (e != cudaSuccess) {
     free_ws(n);
     return e;
@@ -543,68 +540,78 @@ cudaError_t forward(pg_mlp *n, int64_t rows, cudaStream_t st, bool keep) {
 }
 
 // backward from n->dy and n->dyb (gradient of the output in FP32 and BF16,
-// [rows x pout]) into n->g, which it writes whole
+// [rows x pout]) into n->g, which it writes whole.  On tcgen05 the gradient of a
+// hidden layer's pre-activation takes the place of the pre-activation, so that
+// all layers' weight gradients can be formed together at the end.
 cudaError_t backward(pg_mlp *n, int64_t rows, cudaStream_t st) {
   cudaError_t e;
-  bool have_part = false;      // colpart holds the sums of the current gradient
+  const int wmax = std::max(n->width, n->pout);
+  auto is_tc = [&](int l) {
+    return n->use_tc && (n->din[l] == 64 || n->din[l] == 256) &&
+           (n->dout[l] == 64 || n->dout[l] == 256);
+  };
+  std::vector<WeightGrad> wg;
+  const __nv_bfloat16 *dcur = n->dyb;   // gradient of the current pre-activation, BF16
+  bool have_part = false;               // its column sums are in colpart already
   int nparts = 0;
   for (int l = n->nl - 1; l >= 0; --l) {
     const __nv_bfloat16 *X = l == 0 ? n->x0 : n->act[l - 1];
     const int din = n->din[l], dout = n->dout[l];
-    const bool tc = n->use_tc && (din == 64 || din == 256) && (dout == 64 || dout == 256);
+    float *part = n->colpart + (size_t)l * n->col_rows * wmax;
     // bias gradient: column sums of dPre in FP32, from the product that made
     // it or, where that kept no sums, from dy
     if (!have_part) {
       const int64_t per = std::max<int64_t>(64, ((rows + 127) / 128 + 15) / 16 * 16);
       nparts = (int)((rows + per - 1) / per);
       column_sums_part<<<dim3((unsigned)nparts, (unsigned)(dout / 64)), kColThreads, 0, st>>>(
-          n->dy, rows, dout, per, n->colpart);
+          n->dy, rows, dout, per, part);
       note_launches(1);
     }
     // dW [dout x din] = dPre^T X
-    if (tc) {
-      e = gemm_tn_splitk_tc(n->dyb, dout, dout, X, din, din, rows, n->g + n->woff[l], n->gscratch,
-                            n->gscratch_bytes, n->colpart, nparts, n->g + n->boff[l], st, n->d_err);
+    if (is_tc(l)) {
+      wg.push_back(WeightGrad{dcur, X, dout, din, dout, din, n->g + n->woff[l], part, nparts,
+                              n->g + n->boff[l]});
     } else {
-      column_sums_final<<<(dout + 127) / 128, 128, 0, st>>>(n->colpart, nparts, dout,
-                                                            n->g + n->boff[l]);
+      column_sums_final<<<(dout + 127) / 128, 128, 0, st>>>(part, nparts, dout, n->g + n->boff[l]);
       // transposes to K-contiguous [dout x rows], [din x rows]
       dim3 g1((dout + 31) / 32, (unsigned)((rows + 31) / 32));
-      transpose_bf16<<<g1, dim3(32, 8), 0, st>>>(n->dyb, (int)rows, dout, dout, n->dyt, (int)rows);
+      transpose_bf16<<<g1, dim3(32, 8), 0, st>>>(dcur, (int)rows, dout, dout, n->dyt, (int)rows);
       dim3 g2((din + 31) / 32, (unsigned)((rows + 31) / 32));
       transpose_bf16<<<g2, dim3(32, 8), 0, st>>>(X, (int)rows, din, din, n->xt, (int)rows);
       note_launches(3);
       // rows must be a multiple of 32 for the K loop; the batch is padded
-      e = gemm_nt(n->dyt, (int)rows, n->xt, (int)rows, dout, din, (int)rows, nullptr, 0,
-                  n->g + n->woff[l], nullptr, nullptr, din, 0, st);
+      if ((e = gemm_nt(n->dyt, (int)rows, n->xt, (int)rows, dout, din, (int)rows, nullptr, 0,
+                       n->g + n->woff[l], nullptr, nullptr, din, 0, st)) != cudaSuccess)
+        return e;
     }
-    if (e != cudaSuccess) return e;
     if (l == 0) break;
-    if (tc) {
+    __nv_bfloat16 *dprev = n->pre[l - 1];
+    if (is_tc(l)) {
       // dPre of layer l-1 = (dPre W) * GELU'(pre) in one product (B = W^T
-      // [din x dout]), in BF16 into the other buffer (the one read as A must
-      // not be overwritten by other tiles), with its column sums; in FP32 only
-      // for a next layer that goes the other way
-      const int dn = n->din[l - 1];
-      const bool tc_next = (dn == 64 || dn == 256) && (din == 64 || din == 256);
-      if ((e = gemm_nt_tc(n->dyb, dout, n->wbt + n->woff[l], dout, rows, din, dout, nullptr, 2,
-                          tc_next ? nullptr : n->dy, n->dyb2, nullptr, din, st, n->d_err,
-                          n->pre[l - 1], n->colpart, &nparts)) != cudaSuccess)
+      // [din x dout]), each element over the pre-activation it was formed
+      // with, with its column sums; in FP32 only for a next layer that goes
+      // the other way
+      if ((e = gemm_nt_tc(dcur, dout, n->wbt + n->woff[l], dout, rows, din, dout, nullptr, 2,
+                          is_tc(l - 1) ? nullptr : n->dy, dprev, nullptr, din, st, n->d_err, dprev,
+                          n->colpart + (size_t)(l - 1) * n->col_rows * wmax, &nparts)) != cudaSuccess)
         return e;
       have_part = true;
-      std::swap(n->dyb, n->dyb2);
     } else {
       // dX [rows x din] = dPre W  (B = W^T [din x dout])
-      if ((e = gemm_nt(n->dyb, dout, n->wbt + n->woff[l], dout, rows, din, dout, nullptr, 0, n->dy,
+      if ((e = gemm_nt(dcur, dout, n->wbt + n->woff[l], dout, rows, din, dout, nullptr, 0, n->dy,
                        nullptr, nullptr, din, 0, st)) != cudaSuccess)
         return e;
       // through the GELU of layer l-1
-      gelu_backward<<<grid1(rows * din), 256, 0, st>>>(n->dy, n->pre[l - 1], rows, din, n->dyb,
-                                                       n->dy);
+      gelu_backward<<<grid1(rows * din), 256, 0, st>>>(n->dy, dprev, rows, din, dprev, n->dy);
       note_launches(1);
       have_part = false;
     }
+    dcur = dprev;
   }
+  if (!wg.empty() &&
+      (e = gemm_tn_splitk_tc(wg.data(), (int)wg.size(), rows, n->gscratch, n->gscratch_bytes, st,
+                             n->d_err)) != cudaSuccess)
+    return e;
   return cudaGetLastError();
 }
 
@@ -824,9 +831,20 @@ static pg_status mlp_grad_impl(pg_mlp *n, const float *x, const float *t, int64_
   CUM(ensure_ws(n, M));
   pack_input<<<grid1(M * (n->pin / 8)), 256, 0, st>>>(x, M, n->n_in, n->pin, n->x0);
   note_launches(1);
-  CUM(forward(n, M, st, true));
+  // the surrogate's shape in one kernel (16384 rows: five products of 20 us
+  // each, their inputs and weights loaded anew, against 15 us)
+  const bool fused = fused_shape(n);
+  if (fused) {
+    CUM(ensure_packed(n, st));
+    const float *bias[5];
+    for (int l = 0; l < 5; ++l) bias[l] = n->w + n->boff[l];
+    CUM(mlp_fused_forward(x, M, n->n_in, n->wpk, bias, n->y, n->n_out, st, n->d_err, n->pre.data(),
+                          n->act.data()));
+  } else {
+    CUM(forward(n, M, st, true));
+  }
   const int nb = (int)std::min<int64_t>(1024, (M * (n->pout / 8) + 255) / 256);
-  mse_grad<<<nb, 256, 0, st>>>(n->y, n->pout, t, n->n_out, M, n->dy, n->dyb, n->loss_partial);
+  mse_grad<<<nb, 256, 0, st>>>(n->y, fused ? n->n_out : n->pout, n->pout, t, n->n_out, M, n->dy, n->dyb, n->loss_partial);
   note_launches(1);
   CUM(backward(n, M, st));
   if (n->use_tc) {

@@ -2,7 +2,8 @@
 // the 5th-generation tensor cores, activations kept on chip; and, in a
 // second instance of the same kernel, a whole network step of the learned
 // flow map (features gathered from the field, the network, the displacement
-// applied to the particles).
+// applied to the particles), and, in a third, the forward pass of a training
+// batch.
 //
 // Network: 64 (padded input) -> 256 -> 256 -> 256 -> 256 -> n_out (<= 16;
 // the weights are padded to 64 outputs), GELU after the hidden layers (the
@@ -274,7 +275,20 @@ struct FusedArgs {
   int64_t M;
   int n_out;
   int *err;
+  // training: [M x 256] BF16 per hidden layer, before and after GELU
+  __nv_bfloat16 *pre[4], *act[4];
 };
+
+// What an instance of the kernel does: inference, a network step of the flow
+// map, or the forward pass of a training batch (inference that also keeps the
+// hidden layers' values for the backward pass).
+enum : int { FUSED_FORWARD = 0, FUSED_STEP = 1, FUSED_TRAIN = 2 };
+
+__device__ __forceinline__ void store_row32(void *dst, const uint32_t (&w)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n" ::"l"(dst), "r"(w[0]),
+               "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+               : "memory");
+}
 
 // Row m of the FP32 features as 64 BF16 columns, zero beyond n_in and for
 // m >= M.  The loads of a half row are issued together, so one lane keeps 32
@@ -350,23 +364,58 @@ __global__ void __launch_bounds__(128) pack_features_kernel(const __grid_constan
 }
 
 // Bias, GELU and BF16 for 32 columns of a row: v (accumulator values) into
-// four 16-byte chunks of the operand layout.
-__device__ __forceinline__ void gelu_store32(const uint32_t (&v)[32], const float *bias, uint8_t *dst) {
+// four 16-byte chunks of the operand layout; KEEP: and the values before and
+// after GELU to pre and act (32 columns of the row in global memory, null for
+// a row beyond the batch).
+template <bool KEEP>
+__device__ __forceinline__ void gelu_store32(const uint32_t (&v)[32], const float *bias, uint8_t *dst,
+                                             __nv_bfloat16 *pre, __nv_bfloat16 *act) {
+  if constexpr (!KEEP) {
 #pragma unroll
-  for (int cc = 0; cc < 32; cc += 8) {
-    const float4 b0 = __ldg(reinterpret_cast<const float4 *>(bias + cc));
-    const float4 b1 = __ldg(reinterpret_cast<const float4 *>(bias + cc + 4));
-    const float2 bb[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w),
-                          make_float2(b1.x, b1.y), make_float2(b1.z, b1.w)};
-    uint32_t w[4];
+    for (int cc = 0; cc < 32; cc += 8) {
+      const float4 b0 = __ldg(reinterpret_cast<const float4 *>(bias + cc));
+      const float4 b1 = __ldg(reinterpret_cast<const float4 *>(bias + cc + 4));
+      const float2 bb[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w),
+                            make_float2(b1.x, b1.y), make_float2(b1.z, b1.w)};
+      uint32_t w[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float2 x = __fadd2_rn(make_float2(__uint_as_float(v[cc + 2 * j]),
-                                              __uint_as_float(v[cc + 2 * j + 1])), bb[j]);
+      for (int j = 0; j < 4; ++j) {
+        const float2 x = __fadd2_rn(make_float2(__uint_as_float(v[cc + 2 * j]),
+                                                __uint_as_float(v[cc + 2 * j + 1])), bb[j]);
+        const __nv_bfloat162 hv = __float22bfloat162_rn(gelu2_f(x));
+        w[j] = *reinterpret_cast<const uint32_t *>(&hv);
+      }
+      *reinterpret_cast<uint4 *>(dst + (cc >> 3) * 128) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    return;
+  }
+#pragma unroll
+  for (int c16 = 0; c16 < 32; c16 += 16) {
+    uint32_t pw[8], w[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int cc = c16 + 2 * j;
+      const float4 b4 = __ldg(reinterpret_cast<const float4 *>(bias + (cc & ~3)));
+      const float2 x = __fadd2_rn(make_float2(__uint_as_float(v[cc]), __uint_as_float(v[cc + 1])),
+                                  (cc & 2) ? make_float2(b4.z, b4.w) : make_float2(b4.x, b4.y));
+      const __nv_bfloat162 xv = __float22bfloat162_rn(x);
+      pw[j] = *reinterpret_cast<const uint32_t *>(&xv);
       const __nv_bfloat162 hv = __float22bfloat162_rn(gelu2_f(x));
       w[j] = *reinterpret_cast<const uint32_t *>(&hv);
     }
-    *reinterpret_cast<uint4 *>(dst + (cc >> 3) * 128) = make_uint4(w[0], w[1], w[2], w[3]);
+    *reinterpret_cast<uint4 *>(dst + (c16 >> 3) * 128) = make_uint4(w[0], w[1], w[2], w[3]);
+    *reinterpret_cast<uint4 *>(dst + ((c16 >> 3) + 1) * 128) = make_uint4(w[4], w[5], w[6], w[7]);
+    if (pre) {
+      store_row32(pre + c16, pw);
+      // kept as GELU, not twice it
+      const __nv_bfloat162 half = __floats2bfloat162_rn(0.5f, 0.5f);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const __nv_bfloat162 h = __hmul2(*reinterpret_cast<const __nv_bfloat162 *>(&w[j]), half);
+        w[j] = *reinterpret_cast<const uint32_t *>(&h);
+      }
+      store_row32(act + c16, w);
+    }
   }
 }
 
@@ -374,9 +423,10 @@ __device__ __forceinline__ void gelu_store32(const uint32_t (&v)[32], const floa
 // pieces of 32 columns (CPH per 128-column half, from column c0 of each), a
 // piece's values arriving while the one before is worked on.  Two arrivals
 // per half for a warp of a group of eight (CPH 2), one for a warp of sixteen.
-template <int CPH>
+template <int CPH, bool KEEP>
 __device__ __forceinline__ void epilogue_layer(uint32_t tacc, const float *bias, uint8_t *hrow,
-                                               int c0, uint32_t accfree, uint32_t hfull, int lane) {
+                                               int c0, uint32_t accfree, uint32_t hfull, int lane,
+                                               __nv_bfloat16 *pre, __nv_bfloat16 *act) {
   uint32_t v[2][32];
   tmem_ld32(tacc + (uint32_t)c0, v[0]);
 #pragma unroll
@@ -392,7 +442,8 @@ __device__ __forceinline__ void epilogue_layer(uint32_t tacc, const float *bias,
       __syncwarp();
       if (lane == 0) bar_arrive(accfree, CPH);
     }
-    gelu_store32(v[q & 1], bias + col, hrow + (col >> 3) * 128);
+    gelu_store32<KEEP>(v[q & 1], bias + col, hrow + (col >> 3) * 128, KEEP && pre ? pre + col : nullptr,
+                       KEEP && pre ? act + col : nullptr);
     if (q % CPH == CPH - 1) {
       // written by the generic proxy, read by the tensor cores
       asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
@@ -402,11 +453,12 @@ __device__ __forceinline__ void epilogue_layer(uint32_t tacc, const float *bias,
   }
 }
 
-// STEP = false: inference, y = the network on x.  STEP = true: one network
+// FUSED_FORWARD, FUSED_TRAIN: y = the network on x.  FUSED_STEP: one network
 // step of the learned flow map on the particles of a.io, from the packed
 // features a.xpk.
-template <bool STEP>
+template <int MODE>
 __global__ void __launch_bounds__(kFThreads, 1) mlp_fused_kernel(const __grid_constant__ FusedArgs a) {
+  constexpr bool STEP = MODE == FUSED_STEP, KEEP = MODE == FUSED_TRAIN;
   extern __shared__ __align__(1024) uint8_t smem[];
   uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + kOffMisc);
   volatile int *fail = reinterpret_cast<volatile int *>(smem + kOffMisc + 4);
@@ -634,12 +686,17 @@ __global__ void __launch_bounds__(kFThreads, 1) mlp_fused_kernel(const __grid_co
         asm volatile("tcgen05.fence::after_thread_sync;\n");
         if (L < 4) {
           uint8_t *hrow = smem + kOffH + t * kTileHBytes + (r >> 3) * 32 * 128 + (r & 7) * 16;
+          __nv_bfloat16 *pre = nullptr, *act = nullptr;
+          if constexpr (KEEP) {
+            const int64_t m = (t0 + t * G) * TMF + r;
+            if (m < a.M) { pre = a.pre[L] + m * 256; act = a.act[L] + m * 256; }
+          }
           if (nt == 2)
-            epilogue_layer<2>(tacc, a.bias[L], hrow, sub * 64, bar(B_ACCFREE + acc),
-                              bar(B_HFULL + 2 * t), lane);
+            epilogue_layer<2, KEEP>(tacc, a.bias[L], hrow, sub * 64, bar(B_ACCFREE + acc),
+                                    bar(B_HFULL + 2 * t), lane, pre, act);
           else
-            epilogue_layer<1>(tacc, a.bias[L], hrow, sub * 32, bar(B_ACCFREE + acc),
-                              bar(B_HFULL + 2 * t), lane);
+            epilogue_layer<1, KEEP>(tacc, a.bias[L], hrow, sub * 32, bar(B_ACCFREE + acc),
+                                    bar(B_HFULL + 2 * t), lane, pre, act);
         } else {
           const int64_t m0 = (t0 + t * G) * TMF;
           const int rows = (a.M - m0) < TMF ? (int)(a.M - m0) : TMF;
@@ -767,31 +824,49 @@ cudaError_t mlp_fused_pack(const __nv_bfloat16 *const w[5], uint8_t *out, cudaSt
   return cudaGetLastError();
 }
 
-// y [M x n_out] = the network on x [M x n_in] (FP32 features, n_in <= 64,
-// zero-padded to 64 on chip); biases of the five layers (FP32, 256, 256,
-// 256, 256, >= n_out entries); *err (device) set to 1 if a CTA gave up
-// waiting.
-cudaError_t mlp_fused_forward(const float *x, int64_t M, int n_in, const uint8_t *wpk,
-                              const float *const bias[5], float *y, int n_out, cudaStream_t st,
-                              int *err) {
-  if (M == 0) return cudaSuccess;
-  if (n_out < 1 || n_out > 16 || n_in < 1 || n_in > 64 || !err || ((uintptr_t)wpk % 16))
-    return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(mlp_fused_kernel<false>,
+namespace {
+
+template <int MODE>
+cudaError_t launch_fused(FusedArgs &a, const uint8_t *wpk, const float *const bias[5], int n_out,
+                         cudaStream_t st, int *err) {
+  // the attribute belongs to the current device's context: set it on every
+  // launch (cheap), so a first launch on another device is configured too
+  cudaError_t e = cudaFuncSetAttribute(mlp_fused_kernel<MODE>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  FusedArgs a;
-  a.x = x; a.n_in = n_in; a.xpk = nullptr; a.wpk = wpk; a.y = y; a.M = M; a.n_out = n_out;
-  a.err = err;
+  a.wpk = wpk; a.n_out = n_out; a.err = err;
   for (int l = 0; l < 5; ++l) a.bias[l] = bias[l];
-  const int64_t ntiles = (M + TMF - 1) / TMF;
+  const int64_t ntiles = (a.M + TMF - 1) / TMF;
   const int grid = (int)(ntiles < sms ? ntiles : sms);
-  mlp_fused_kernel<false><<<grid, kFThreads, kSmem, st>>>(a);
+  mlp_fused_kernel<MODE><<<grid, kFThreads, kSmem, st>>>(a);
   note_launches(1);
   return cudaGetLastError();
+}
+
+}  // namespace
+
+// y [M x n_out] = the network on x [M x n_in] (FP32 features, n_in <= 64,
+// zero-padded to 64 on chip); biases of the five layers (FP32, 256, 256,
+// 256, 256, >= n_out entries); pre, act (both null, or four [M x 256] BF16
+// arrays each, 32-byte aligned): the hidden layers' values before and after
+// GELU, for a backward pass; *err (device) set to 1 if a CTA gave up waiting.
+cudaError_t mlp_fused_forward(const float *x, int64_t M, int n_in, const uint8_t *wpk,
+                              const float *const bias[5], float *y, int n_out, cudaStream_t st,
+                              int *err, __nv_bfloat16 *const *pre, __nv_bfloat16 *const *act) {
+  if (M == 0) return cudaSuccess;
+  if (n_out < 1 || n_out > 16 || n_in < 1 || n_in > 64 || !err || ((uintptr_t)wpk % 16))
+    return cudaErrorInvalidValue;
+  FusedArgs a{};
+  a.x = x; a.n_in = n_in; a.y = y; a.M = M;
+  if (!pre) return launch_fused<FUSED_FORWARD>(a, wpk, bias, n_out, st, err);
+  for (int l = 0; l < 4; ++l) {
+    if (((uintptr_t)pre[l] | (uintptr_t)act[l]) % 32) return cudaErrorInvalidValue;
+    a.pre[l] = pre[l]; a.act[l] = act[l];
+  }
+  return launch_fused<FUSED_TRAIN>(a, wpk, bias, n_out, st, err);
 }
 
 // Bytes of the packed input tiles of a network step on n particles.
@@ -808,22 +883,12 @@ cudaError_t mlp_fused_step_launch(const SurrogateStepIO &io, uint8_t *xpk, const
   if (io.n == 0) return cudaSuccess;
   if (!err || !io.ferr || !xpk || (((uintptr_t)wpk | (uintptr_t)xpk) % 16))
     return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(mlp_fused_kernel<true>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-  if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  FusedArgs a;
-  a.x = nullptr; a.n_in = kSurFeat; a.io = io; a.xpk = xpk; a.wpk = wpk; a.y = nullptr;
-  a.M = io.n; a.n_out = 3; a.err = err;
-  for (int l = 0; l < 5; ++l) a.bias[l] = bias[l];
+  FusedArgs a{};
+  a.n_in = kSurFeat; a.io = io; a.xpk = xpk; a.M = io.n;
   const int64_t ntiles = (io.n + TMF - 1) / TMF;
-  const int grid = (int)(ntiles < sms ? ntiles : sms);
   pack_features_kernel<<<(unsigned)ntiles, TMF, 0, st>>>(io, ntiles * TMF, xpk);
-  mlp_fused_kernel<true><<<grid, kFThreads, kSmem, st>>>(a);
-  note_launches(2);
-  return cudaGetLastError();
+  note_launches(1);
+  return launch_fused<FUSED_STEP>(a, wpk, bias, 3, st, err);
 }
 
 }  // namespace pg

@@ -90,10 +90,11 @@ __device__ __forceinline__ void store32(void *dst, const uint32_t (&w)[8]) {
                : "memory");
 }
 __device__ __forceinline__ void load32(const void *src, uint32_t (&w)[8]) {
-  asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+  asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
                : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]),
                  "=r"(w[6]), "=r"(w[7])
-               : "l"(src));
+               : "l"(src)
+               : "memory");
 }
 
 // 16 FP32 values rounded to BF16 (nearest even, in pairs), one 32-byte store.
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 gemm_tc_kernel(const __nv_bfloat16 *__restrict__ A, int lda, const __nv_bfloat16 *__restrict__ B,
                int ldb, int64_t M, const float *__restrict__ bias, int act, float *out_f32,
                __nv_bfloat16 *out_bf16, __nv_bfloat16 *pre_bf16,
-               const __nv_bfloat16 *__restrict__ gin, int ldc, float *colpart, int *err) {
+               const __nv_bfloat16 *gin, int ldc, float *colpart, int *err) {
   constexpr int NCOLS = N < 32 ? 32 : N;       // TMEM columns (power of two >= 32)
   constexpr uint32_t SB = N * K * 2, SA = TM * K * 2;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -362,7 +363,8 @@ int gemm_tc_max_ctas() {
 // Products of the MLP on tcgen05; N and K must be 64 or 256, all row
 // strides multiples of 8 elements (ldc of 16), bias 16-byte and outputs 32-byte
 // aligned.
-// colpart (may be null): column sums of the result over each CTA's rows,
+// out_bf16 may be gin: an element is read before it is written, by the same
+// thread.  colpart (may be null): column sums of the result over each CTA's rows,
 // [*nparts][N] FP32, from the values before they are rounded to BF16.  *err
 // (device) is set to 1 if a CTA gave up waiting for its accumulator.
 cudaError_t gemm_nt_tc(const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, int ldb,
@@ -419,19 +421,36 @@ __device__ __forceinline__ void load_chunk_mn(uint8_t *dst, const __nv_bfloat16 
   }
 }
 
-// CTA (m-tile mt, split s): D_s = A[K slice, mt columns]^T . B[K slice, :] in
-// TMEM over chunks [c0, c1) through a ring of kStages buffers (the four
-// chunks of a 64-way split of 16384 rows are all in flight at once), then
-// the FP32 partial [128 x N] to part[s][mt * 128 + row][col].
+// The weight gradients of one or more layers in one launch.  Group g (a layer)
+// has mtiles * splits CTAs from CTA `first`; CTA (m-tile mt, split s) forms D_s
+// = A[K slice, mt columns]^T . B[K slice, :] in TMEM over chunks [c0, c1)
+// through a ring of kStages buffers, then the FP32 partial [128 x N] to
+// part[s][mt * 128 + row][col].  All layers together, because one layer's
+// products fill the chip only when they are cut into 64 splits whose partials
+// cost as much again to write and sum (16384 rows: five launches and five sums
+// 88 us, one of each 25).
 constexpr int kStages = 4;
+constexpr int kMaxGroups = 20;
+struct SplitGroup {
+  const __nv_bfloat16 *A, *B;
+  int64_t lda, ldb;
+  int Mrows, N, mtiles, first;
+  float *part, *out;
+  const float *bpart;
+  int nparts, rblock;          // rblock: first block of its sums
+  float *bout;
+};
+struct SplitGroups {
+  SplitGroup g[kMaxGroups];
+  int n, cps, splits;
+  int64_t K;
+  int *err;
+};
 
-template <int N>
 __global__ void __launch_bounds__(kTcThreads, 1)
-gemm_splitk_tc_kernel(const __nv_bfloat16 *__restrict__ A, int64_t lda, int Mrows,
-                      const __nv_bfloat16 *__restrict__ B, int64_t ldb, int64_t K, int cps,
-                      int mtiles, float *part, int *err) {
-  constexpr int NCOLS = N < 32 ? 32 : N;
-  constexpr uint32_t SA = TM * KC * 2, SB = N * KC * 2;
+gemm_splitk_tc_kernel(const __grid_constant__ SplitGroups args) {
+  constexpr int NCOLS = 256;
+  constexpr uint32_t SA = TM * KC * 2, SB = NCOLS * KC * 2;
   extern __shared__ __align__(1024) uint8_t smem[];
   // stage st: A at smem + st * (SA + SB), B behind it
   auto sA = [&](int st) { return smem + st * (SA + SB); };
@@ -439,20 +458,26 @@ gemm_splitk_tc_kernel(const __nv_bfloat16 *__restrict__ A, int64_t lda, int Mrow
   uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + kStages * (SA + SB));
   uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + kStages * (SA + SB) + kStages * 8);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int mt = blockIdx.x % mtiles, sp = blockIdx.x / mtiles;
-  const int64_t nchunks = (K + KC - 1) / KC;
-  const int64_t c0 = (int64_t)sp * cps;
-  const int64_t c1 = c0 + cps < nchunks ? c0 + cps : nchunks;
-  const int rows = Mrows - mt * TM < TM ? Mrows - mt * TM : TM;
-  const __nv_bfloat16 *Am = A + (size_t)mt * TM;
+  int gi = 0;
+  while (gi + 1 < args.n && (int)blockIdx.x >= args.g[gi + 1].first) ++gi;
+  const SplitGroup &G = args.g[gi];
+  const int N = G.N, local = (int)blockIdx.x - G.first;
+  const int mt = local % G.mtiles, sp = local / G.mtiles, mtiles = G.mtiles;
+  const int64_t K = args.K, nchunks = (K + KC - 1) / KC;
+  const int64_t c0 = (int64_t)sp * args.cps;
+  const int64_t c1 = c0 + args.cps < nchunks ? c0 + args.cps : nchunks;
+  const int rows = G.Mrows - mt * TM < TM ? G.Mrows - mt * TM : TM;
+  const __nv_bfloat16 *Am = G.A + (size_t)mt * TM;
+  int *err = args.err;
 
   // one copy group per chunk, empty past the last one, so that group counts
   // and chunks agree
   auto copy_chunk = [&](int64_t c) {
     if (c < c1) {
       const int st = (int)((c - c0) % kStages);
-      load_chunk_mn<TM / 8>(sA(st), Am, lda, rows, c * KC, K);
-      load_chunk_mn<N / 8>(sB(st), B, ldb, N, c * KC, K);
+      load_chunk_mn<TM / 8>(sA(st), Am, G.lda, rows, c * KC, K);
+      if (N == 256) load_chunk_mn<32>(sB(st), G.B, G.ldb, N, c * KC, K);
+      else load_chunk_mn<8>(sB(st), G.B, G.ldb, N, c * KC, K);
     }
     asm volatile("cp.async.commit_group;\n");
   };
@@ -496,7 +521,7 @@ gemm_splitk_tc_kernel(const __nv_bfloat16 *__restrict__ A, int64_t lda, int Mrow
       for (int ks = 0; ks < KC / 16; ++ks) {
         // two row groups of 8 per product: leading offset between them
         const uint64_t da = smem_desc(su32(sA(st)) + ks * 2 * TM * 16, TM * 16, 128);
-        const uint64_t db = smem_desc(su32(sB(st)) + ks * 2 * N * 16, N * 16, 128);
+        const uint64_t db = smem_desc(su32(sB(st)) + (uint32_t)(ks * 2 * N * 16), (uint32_t)N * 16, 128);
         const uint32_t accum = (c > c0 || ks > 0) ? 1u : 0u;
         asm volatile(
             "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
@@ -524,7 +549,7 @@ gemm_splitk_tc_kernel(const __nv_bfloat16 *__restrict__ A, int64_t lda, int Mrow
   } else if (last_stage >= 0) {
     asm volatile("tcgen05.fence::after_thread_sync;\n");
     const int lg = warp & 3;
-    float *out = part + ((size_t)sp * mtiles * TM + (size_t)mt * TM + lg * 32 + lane) * N;
+    float *out = G.part + ((size_t)sp * mtiles * TM + (size_t)mt * TM + lg * 32 + lane) * N;
 #pragma unroll 1
     for (int cc = (warp >> 2) * 16; cc < N; cc += 16 * kColGroups) {
       uint32_t r[16];
@@ -552,88 +577,99 @@ gemm_splitk_tc_kernel(const __nv_bfloat16 *__restrict__ A, int64_t lda, int Mrow
   }
 }
 
-// out[q] = sum over splits s of part[s][q], q < total; and, for the layer's
-// bias gradient, bout[c] = sum over p of bpart[p][c], c < nb.  A block takes
-// 64 outputs side by side; its four groups of 64 threads each sum a quarter
-// of the partials in order, and the quarters are added in order (fixed order,
-// so the result does not depend on timing).  Four quarters instead of one
-// chain: the loads of 64 to 152 partials are the time here.
+// Of each group: out[q] = sum over splits s of part[s][q], and, for the
+// layer's bias gradient, bout[c] = sum over p of bpart[p][c].  A block takes 64
+// outputs side by side; its four groups of 64 threads each sum a quarter of
+// the partials in order, and the quarters are added in order (fixed order, so
+// the result does not depend on timing).  Four quarters instead of one chain:
+// the loads of up to 152 partials are the time here.
 constexpr int kRedOut = 64;
-__global__ void __launch_bounds__(256) splitk_reduce_kernel(
-    const float *part, int splits, size_t stride, int total, float *out, const float *bpart,
-    int nparts, int nb, float *bout) {
+__global__ void __launch_bounds__(256) splitk_reduce_kernel(const __grid_constant__ SplitGroups args) {
   __shared__ float sh[4][kRedOut];
+  int gi = 0;
+  while (gi + 1 < args.n && (int)blockIdx.x >= args.g[gi + 1].rblock) ++gi;
+  const SplitGroup &G = args.g[gi];
   const int lane = threadIdx.x & (kRedOut - 1), quarter = threadIdx.x / kRedOut;
-  const int wblocks = total / kRedOut;
-  const bool bias = (int)blockIdx.x >= wblocks;
-  const float *src = bias ? bpart : part;
-  const int q = (bias ? (int)blockIdx.x - wblocks : (int)blockIdx.x) * kRedOut + lane;
-  const int n = bias ? nparts : splits;
-  const size_t step = bias ? (size_t)nb : stride;
+  const int blk = (int)blockIdx.x - G.rblock, wblocks = G.Mrows * G.N / kRedOut;
+  const bool bias = blk >= wblocks;
+  const float *src = bias ? G.bpart : G.part;
+  const int q = (bias ? blk - wblocks : blk) * kRedOut + lane;
+  const int n = bias ? G.nparts : args.splits;
+  const size_t step = bias ? (size_t)G.Mrows : (size_t)G.mtiles * TM * G.N;
   const int per = (n + 3) / 4, s1 = min(n, (quarter + 1) * per);
   float acc = 0.f;
-#pragma unroll 16
+#pragma unroll 8
   for (int s = quarter * per; s < s1; ++s) acc += src[(size_t)s * step + q];
   sh[quarter][lane] = acc;
   __syncthreads();
   if (quarter == 0) {
     const float v = (sh[0][lane] + sh[1][lane]) + (sh[2][lane] + sh[3][lane]);
-    if (bias) bout[q] = v;
-    else out[q] = v;
+    if (bias) G.bout[q] = v;
+    else G.out[q] = v;
   }
 }
 
-template <int N>
-cudaError_t launch_splitk(const __nv_bfloat16 *A, int64_t lda, int Mrows, const __nv_bfloat16 *B,
-                          int64_t ldb, int64_t K, float *out, float *scratch, size_t scratch_bytes,
-                          const float *bpart, int nparts, float *bout, cudaStream_t st, int *err) {
-  constexpr size_t smem = kStages * ((size_t)TM * KC * 2 + (size_t)N * KC * 2 + 8) + 16;
-  cudaError_t e = cudaFuncSetAttribute(gemm_splitk_tc_kernel<N>,
+}  // namespace
+
+// Weight and bias gradients of `ng` layers on tcgen05, one launch and one of
+// sums: for each, out[Mrows x N] (FP32, row-major) = A^T B with A [K x Mrows]
+// and B [K x N] BF16 row-major (row strides lda, ldb, multiples of 8), K (the
+// batch) any number of rows, N 64 or 256, Mrows 64 or 256; bout[Mrows] = the
+// sum of the nparts rows of bpart (column-sum partials of A's FP32 values).
+// The K range is split over CTAs; each writes an FP32 partial to `scratch`
+// and a fixed-order sum reduces them (deterministic).  The operands are read
+// MN-major, so the batch needs no transposed copies (16384 rows: ten
+// transposes were 100 us of a pass).  *err (device) is set to 1 if a CTA gave
+// up waiting for its products.
+cudaError_t gemm_tn_splitk_tc(const WeightGrad *w, int ng, int64_t K, float *scratch,
+                              size_t scratch_bytes, cudaStream_t st, int *err) {
+  if (K == 0 || ng == 0) return cudaSuccess;
+  if (ng < 0 || ng > kMaxGroups || !err || ((uintptr_t)scratch % 32)) return cudaErrorInvalidValue;
+  SplitGroups a;
+  a.n = ng; a.K = K; a.err = err;
+  int mtiles = 0, rblocks = 0;
+  size_t per_split = 0;
+  for (int i = 0; i < ng; ++i) {
+    if (w[i].lda % 8 || w[i].ldb % 8 || (w[i].Mrows != 64 && w[i].Mrows != 256) ||
+        (w[i].N != 64 && w[i].N != 256) || !w[i].bpart || !w[i].bout ||
+        (((uintptr_t)w[i].A | (uintptr_t)w[i].B) % 16))
+      return cudaErrorInvalidValue;
+    SplitGroup &g = a.g[i];
+    g.A = w[i].A; g.B = w[i].B; g.lda = w[i].lda; g.ldb = w[i].ldb;
+    g.Mrows = w[i].Mrows; g.N = w[i].N;
+    g.mtiles = (w[i].Mrows + TM - 1) / TM;
+    g.out = w[i].out; g.bpart = w[i].bpart; g.nparts = w[i].nparts; g.bout = w[i].bout;
+    g.rblock = rblocks;
+    rblocks += (g.Mrows * g.N + g.Mrows) / kRedOut;
+    mtiles += g.mtiles;
+    per_split += (size_t)g.mtiles * TM * g.N;
+  }
+  constexpr size_t smem = kStages * ((size_t)TM * KC * 2 + (size_t)256 * KC * 2 + 8) + 16;
+  cudaError_t e = cudaFuncSetAttribute(gemm_splitk_tc_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int mtiles = (Mrows + TM - 1) / TM;
+  // as many splits as give every multiprocessor a CTA
   const int64_t nchunks = (K + KC - 1) / KC;
-  const size_t per_split = (size_t)mtiles * TM * N * sizeof(float);
   int64_t want = std::max<int64_t>(1, std::min<int64_t>(nchunks, (int64_t)sms / mtiles));
-  want = std::min<int64_t>(want, (int64_t)(scratch_bytes / per_split));
+  want = std::min<int64_t>(want, (int64_t)(scratch_bytes / (per_split * sizeof(float))));
   if (want < 1) return cudaErrorInvalidValue;
-  const int cps = (int)((nchunks + want - 1) / want);
-  const int splits = (int)((nchunks + cps - 1) / cps);
-  gemm_splitk_tc_kernel<N><<<splits * mtiles, kTcThreads, smem, st>>>(A, lda, Mrows, B, ldb, K,
-                                                                       cps, mtiles, scratch, err);
-  // Mrows and N are 64 or 256: whole blocks of kRedOut outputs
-  splitk_reduce_kernel<<<(Mrows * N + Mrows) / kRedOut, 256, 0, st>>>(
-      scratch, splits, (size_t)mtiles * TM * N, Mrows * N, out, bpart, nparts, Mrows, bout);
+  a.cps = (int)((nchunks + want - 1) / want);
+  a.splits = (int)((nchunks + a.cps - 1) / a.cps);
+  int first = 0;
+  float *part = scratch;
+  for (int i = 0; i < ng; ++i) {
+    a.g[i].first = first;
+    a.g[i].part = part;
+    first += a.splits * a.g[i].mtiles;
+    part += (size_t)a.splits * a.g[i].mtiles * TM * a.g[i].N;
+  }
+  gemm_splitk_tc_kernel<<<first, kTcThreads, smem, st>>>(a);
+  splitk_reduce_kernel<<<rblocks, 256, 0, st>>>(a);
   note_launches(2);
   return cudaGetLastError();
-}
-
-}  // namespace
-
-// Weight and bias gradient of a layer on tcgen05: out[Mrows x N] (FP32,
-// row-major) = A^T B with A [K x Mrows] and B [K x N] BF16 row-major (row
-// strides lda, ldb, multiples of 8), K (the batch) any number of rows, N 64
-// or 256, Mrows 64 or 256; bout[Mrows] = the sum of the nparts rows of bpart
-// (column-sum partials of A's FP32 values).  The K range is split over CTAs;
-// each writes an FP32 partial to `scratch` and a fixed-order sum reduces them
-// (deterministic).  The operands are read MN-major, so the batch needs no
-// transposed copies (16384 rows: ten transposes were 100 us of a pass).  *err
-// (device) is set to 1 if a CTA gave up waiting for its products.
-cudaError_t gemm_tn_splitk_tc(const __nv_bfloat16 *A, int64_t lda, int Mrows,
-                              const __nv_bfloat16 *B, int64_t ldb, int N, int64_t K, float *out,
-                              float *scratch, size_t scratch_bytes, const float *bpart, int nparts,
-                              float *bout, cudaStream_t st, int *err) {
-  if (K == 0 || Mrows == 0) return cudaSuccess;
-  if (lda % 8 || ldb % 8 || !err || (Mrows != 64 && Mrows != 256) || ((uintptr_t)scratch % 32) ||
-      !bpart || !bout)
-    return cudaErrorInvalidValue;
-  if (((uintptr_t)A | (uintptr_t)B) % 16) return cudaErrorInvalidValue;
-  if (N == 256) return launch_splitk<256>(A, lda, Mrows, B, ldb, K, out, scratch, scratch_bytes, bpart, nparts, bout, st, err);
-  if (N == 64) return launch_splitk<64>(A, lda, Mrows, B, ldb, K, out, scratch, scratch_bytes, bpart, nparts, bout, st, err);
-  return cudaErrorNotSupported;
 }
 
 }  // namespace pg

@@ -227,6 +227,16 @@ struct SurrogateStepIO {
   double horizon;
   int *ferr;                  // device word: feature error (time range, missing slab)
 };
+// A layer's weight and bias gradient (gemm_tn_splitk_tc, mlp_tc.cu).
+struct WeightGrad {
+  const __nv_bfloat16 *A, *B;   // [batch x Mrows], [batch x N]
+  int64_t lda, ldb;
+  int Mrows, N;
+  float *out;                   // [Mrows x N]
+  const float *bpart;           // [nparts x Mrows]
+  int nparts;
+  float *bout;                  // [Mrows]
+};
 // Whether the network's engine and shape allow the fused step.
 bool mlp_fused_step_ok(const pg_mlp *net);
 // Bytes of the packed features of a step on n particles.

@@ -244,3 +244,22 @@ def test_fused_forward_with_lone_and_paired_tiles(gpu, tiles, extra):
         got = net.forward(x)
         assert torch.equal(got, want)
         assert torch.equal(net.forward(x), got)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M", [32, 160, 128 * 152, 128 * 152 + 32, 128 * 320])
+def test_fused_training_forward_keeps_the_layers_values(gpu, M):
+    """The gradient from the forward pass in one kernel equals the one from the
+    layer-by-layer forward bit for bit (the same values before and after
+    GELU, the same backward): part of a tile, tiles alone and in pairs."""
+    pg, torch = gpu
+    net = pg.MLP(37, 256, 4, 3, seed=19)
+    g = torch.Generator("cuda").manual_seed(M)
+    x = torch.randn(M, 37, device="cuda", generator=g)
+    t = torch.randn(M, 3, device="cuda", generator=g)
+    net.set_engine(2)
+    loss, want = net.grad(x, t)
+    net.set_engine(1)
+    loss1, got = net.grad(x, t)
+    assert loss1 == loss
+    np.testing.assert_array_equal(got, want)
