@@ -359,9 +359,9 @@ __device__ __forceinline__ bool corner_offsets(const A &a, const Sampler<Real, S
     atomicCAS(a.err, 0, (int)DEVERR_CELL_INDEX);
     return false;
   }
-  const unsigned row = (D3 ? (unsigned)c.ck * (unsigned)g.ny : 0u) + (unsigned)c.cj;
-  o.first = ((size_t)row * (unsigned)g.nx + (unsigned)c.ci) * EB;
-  o.dx = (ptrdiff_t)((c.ci + 1 == g.nx ? 1 - g.nx : 1) * EB);
+  const size_t row = (D3 ? (size_t)(unsigned)c.ck * (unsigned)g.ny : 0) + (unsigned)c.cj;
+  o.first = (row * (unsigned)g.nx + (unsigned)c.ci) * EB;
+  o.dx = (ptrdiff_t)(c.ci + 1 == g.nx ? 1 - g.nx : 1) * EB;
   o.dy = (size_t)(unsigned)g.nx * EB;
   o.dz = o.dy * (unsigned)g.ny;
   return true;

@@ -1273,14 +1273,15 @@ pg_status pg_execute_records(pg_pset *ps, const pg_kernel *k, double runtime, do
 // location and corner gather of each particle, and a small set is at rest
 // between launches, so launches are long (1440 steps; 38 launches of 64 took
 // 100 particles 2.7 ms for 2400 steps) -- but only where their length cannot
-// show in the results: the FP32 forms keep a step's time as an FP32 offset in
-// its snapshot interval, advanced step by step and formed anew at each
-// launch, which is exact while times, steps and interval are whole seconds
-// below 2^24.  Anything else keeps 64.
+// show in the results: the FP32 forms count a launch's steps from its start
+// time, and keep a step's time as an FP32 offset in its snapshot interval,
+// advanced step by step and formed anew at each launch, which is exact while
+// times, steps and interval are whole seconds below 2^24.  Anything else
+// keeps 64.
 static int default_chunk(const pg_pset *ps, const pg_kernel *k, double dt) {
   const pg_fieldset *fs = ps->fs;
   constexpr int kLong = 1440, kShort = 64;
-  if (ps->pos == PG_POS_F64 || fs->nt == 1 || k->scheme == PG_RKF45) return kLong;
+  if (ps->pos == PG_POS_F64 || k->scheme == PG_RKF45) return kLong;
   auto whole = [](double v) { return std::fabs(v) < 9.0e15 && v == std::floor(v); };
   if (!whole(dt) || ps->t_min != ps->t_max || !whole(ps->t_min) || !whole(fs->period)) return kShort;
   double gap = fs->period > 0.0 ? fs->times[0] + fs->period - fs->times.back() : 0.0;

@@ -141,3 +141,35 @@ def test_backward_streamed_equals_resident(pg, ring):
         res.append(gpu_run(ps, pg.Kernel("rk4"), 4.5 * DAY, -1800.0, 2.25 * DAY))
     for k in ("lon", "lat", "depth", "status", "time", "step"):
         np.testing.assert_array_equal(res[1]["final"][k], res[0]["final"][k], err_msg=k)
+
+
+@pytest.mark.parametrize("dt", [1800.0, 1234.5])
+@pytest.mark.parametrize("pos,storage,n", [("f32", "f32", 1), ("f32", "f32", 1217), ("f32", "f32", 9729),
+                                           ("cell", "f16", 300), ("cell", "f16", 2433),
+                                           ("f64", "f64", 152), ("f64", "f64", 153)])
+def test_small_sets_and_default_launches_equal_full_warps_and_short_ones(pg, pos, storage, n, dt):
+    """A small set (fewer particles per warp; counts around the limits of a
+    152-multiprocessor chip) gives each particle the result it has in a set
+    of full warps, and launches of the default length that of 64-step ones,
+    for whole and fractional steps."""
+    rng = np.random.default_rng(n)
+    nx, ny = 24, 13
+    spec = synth.FieldSpec(np.arange(nx) * 15.0, -45.0 + 7.5 * np.arange(ny), np.zeros(1),
+                           np.arange(3) * DAY, rng.normal(size=(3, 2, 1, ny, nx)) * 3.0, 1, True,
+                           3 * DAY, 2, None)
+    fs = pg.FieldSet.from_spec(spec, storage=storage)
+    big = 40_000
+    lon = rng.uniform(0.0, 360.0, big).astype(np.float32).astype(np.float64)
+    lat = rng.uniform(-30.0, 30.0, big).astype(np.float32).astype(np.float64)
+    k = pg.Kernel("rk4", ("brownian",), kh=10.0)
+
+    def run(m, chunk):
+        ps = pg.ParticleSet(fs, lon[:m], lat[:m], pos=pos, seed=3)
+        if chunk:
+            ps.set_tune(block=128, resort_steps=0, chunk_steps=chunk)
+        ps.execute(k, 100 * dt, dt)
+        return ps.get()
+    small, short, full = run(n, 0), run(n, 64), run(big, 64)
+    for key in ("lon", "lat", "time", "step", "status"):
+        np.testing.assert_array_equal(small[key], short[key], err_msg=key)
+        np.testing.assert_array_equal(small[key], full[key][:n], err_msg=key)
