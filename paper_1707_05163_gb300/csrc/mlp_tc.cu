@@ -16,13 +16,20 @@
 // because the piece loop is a chain of waits (tensor memory, the stored
 // pre-activation).  A gradient of 16384 rows of the surrogate network took
 // 3154 us with serial column sums, ten transposed copies and four-warp
-// epilogues, and takes 339 us.
+// epilogues, and takes 189 us (with a fused forward and grouped weight
+// gradients).
 //
-// Shared-memory operand layout (K-major, no swizzle): 8-row x 16-byte core
-// matrices; core matrix (row group g, 16-byte K chunk c) sits at byte
-// (g * K/8 + c) * 128, so neighbouring K chunks are 128 bytes apart (the
-// descriptor's leading-dimension offset) and neighbouring row groups K/8 *
-// 128 bytes apart (its stride-dimension offset).
+// Shared-memory operand layout: 128-byte swizzle, 1024-byte atoms of eight rows
+// of 128 bytes whose 16-byte chunk c of row r sits in place c ^ (r % 8).
+// K-major (gemm_tc_kernel): an atom is 8 rows x 64 K; atoms of neighbouring
+// row groups are 1024 bytes apart (the descriptor's stride offset), K blocks
+// of 64 follow one another.  MN-major (the weight gradient): an atom is 8 K x
+// 64 columns; neighbouring K groups are 1024 bytes apart (stride offset), the
+// next 64 columns KC * 128 bytes (leading offset).  Lanes then copy along a
+// row, 128 to 512 contiguous bytes, and eight of them fill a row of an atom,
+// all banks once.  (Unswizzled core matrices want eight rows per eight lanes:
+// 16 bytes of each: a gradient of 16384 rows took 228 us, of 65536 rows 549
+// us, against 189 and 441.)
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -65,14 +72,21 @@ __device__ __forceinline__ float gelu_grad_tc(float x) {
 }
 
 // 64-bit shared-memory matrix descriptor: start address, leading and stride
-// byte offsets (all >> 4), the fixed 0b001 at bits 46-48, no swizzle.
+// byte offsets (all >> 4), the fixed 0b001 at bits 46-48, 128-byte swizzle (2
+// at bits 61-63).
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
   uint64_t d = 0;
   d |= (uint64_t)((addr & 0x3FFFF) >> 4);
   d |= (uint64_t)((lbo & 0x3FFFF) >> 4) << 16;
   d |= (uint64_t)((sbo & 0x3FFFF) >> 4) << 32;
   d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
   return d;
+}
+
+// Byte offset of 16-byte chunk c of row r in a swizzled atom column.
+__device__ __forceinline__ uint32_t swizzled(int r, int c) {
+  return (uint32_t)((r >> 3) * 1024 + (r & 7) * 128 + (((c & 7) ^ (r & 7)) << 4));
 }
 
 // Instruction descriptor, kind::f16: D FP32, A and B BF16, both K-major.
@@ -136,20 +150,15 @@ __device__ __forceinline__ float warp_column_sums16(float (&v)[16], int lane) {
   return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
-// copy rows [0, rows) of a K-wide BF16 matrix (row stride ld) into the
-// core-matrix layout; rows in [rows, R) are zero-filled (R a multiple of 8).
-// Eight lanes take the eight rows of a core matrix, 128 contiguous bytes of
-// shared memory, and the warp four neighbouring chunks, 64 bytes of each row.
-// (Lanes along a row would write at a stride of 128 bytes, all to the same
-// banks: 6 us of a 256 x 256 product's 23.)
+// copy rows [0, rows) of a K-wide BF16 matrix (row stride ld) into the K-major
+// layout; rows in [rows, R) are zero-filled (R a multiple of 8)
 template <int K>
 __device__ __forceinline__ void load_tile(uint8_t *dst, const __nv_bfloat16 *src, int ld, int rows,
                                           int R) {
   constexpr int KC = K / 8;   // 16-byte chunks per row
   for (int idx = threadIdx.x; idx < R * KC; idx += kTcThreads) {
-    const int r8 = idx & 7, c = (idx >> 3) % KC, g = (idx >> 3) / KC;
-    const int r = g * 8 + r8;
-    const uint32_t off = (uint32_t)((g * KC + c) * 128 + r8 * 16);
+    const int r = idx / KC, c = idx % KC;
+    const uint32_t off = (uint32_t)((c >> 3) * (R * 128)) + swizzled(r, c);
     const bool ok = r < rows;
     const __nv_bfloat16 *s = src + (size_t)(ok ? r : 0) * ld + c * 8;
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(su32(dst + off)),
@@ -227,8 +236,9 @@ gemm_tc_kernel(const __nv_bfloat16 *__restrict__ A, int lda, const __nv_bfloat16
       asm volatile("tcgen05.fence::after_thread_sync;\n");
 #pragma unroll
       for (int ks = 0; ks < K / 16; ++ks) {
-        const uint64_t da = smem_desc(su32(sA) + ks * 256, 128, (K / 8) * 128);
-        const uint64_t db = smem_desc(su32(sB) + ks * 256, 128, (K / 8) * 128);
+        // 16 K-columns: 32 bytes along an atom's rows, four to a K block
+        const uint64_t da = smem_desc(su32(sA) + (ks >> 2) * (TM * 128) + (ks & 3) * 32, 16, 1024);
+        const uint64_t db = smem_desc(su32(sB) + (ks >> 2) * (N * 128) + (ks & 3) * 32, 16, 1024);
         asm volatile(
             "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
             " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
@@ -401,19 +411,15 @@ __host__ __device__ constexpr uint32_t instr_desc_mn(int m, int n) {
 }
 
 // copy batch rows [k0, k0 + KC) of columns [0, cols) of a BF16 matrix (row
-// stride ld, K valid rows) into MN-major core matrices of 8 rows (K) x 16
-// bytes (8 columns): core (row group g, column chunk c) at byte (g * CC + c) *
-// 128, so neighbouring column chunks are 128 bytes apart (the descriptor's
-// stride offset) and neighbouring row groups CC * 128 (its leading offset);
-// columns >= cols and rows >= K are zero-filled.  Eight lanes take the eight
-// rows of a core (distinct banks), four neighbouring chunks 64 bytes of a row.
+// stride ld, K valid rows, CC chunks of 8 columns) into the MN-major layout;
+// columns >= cols and rows >= K are zero-filled
 template <int CC>
 __device__ __forceinline__ void load_chunk_mn(uint8_t *dst, const __nv_bfloat16 *src, int64_t ld,
                                               int cols, int64_t k0, int64_t K) {
   for (int idx = threadIdx.x; idx < KC * CC; idx += kTcThreads) {
-    const int r = idx & 7, c = (idx >> 3) % CC, g = (idx >> 3) / CC;
-    const uint32_t off = (uint32_t)((g * CC + c) * 128 + r * 16);
-    const int64_t m = k0 + g * 8 + r;
+    const int c = idx % CC, k = idx / CC;
+    const uint32_t off = (uint32_t)((c >> 3) * (KC * 128)) + swizzled(k, c);
+    const int64_t m = k0 + k;
     const bool ok = m < K && c * 8 < cols;
     const __nv_bfloat16 *s = src + (ok ? (size_t)m * ld + (size_t)c * 8 : 0);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(su32(dst + off)),
@@ -519,9 +525,9 @@ gemm_splitk_tc_kernel(const __grid_constant__ SplitGroups args) {
       asm volatile("tcgen05.fence::after_thread_sync;\n");
 #pragma unroll
       for (int ks = 0; ks < KC / 16; ++ks) {
-        // two row groups of 8 per product: leading offset between them
-        const uint64_t da = smem_desc(su32(sA(st)) + ks * 2 * TM * 16, TM * 16, 128);
-        const uint64_t db = smem_desc(su32(sB(st)) + (uint32_t)(ks * 2 * N * 16), (uint32_t)N * 16, 128);
+        // 16 batch rows: two K groups of an atom column
+        const uint64_t da = smem_desc(su32(sA(st)) + ks * 2048, KC * 128, 1024);
+        const uint64_t db = smem_desc(su32(sB(st)) + ks * 2048, KC * 128, 1024);
         const uint32_t accum = (c > c0 || ks > 0) ? 1u : 0u;
         asm volatile(
             "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
