@@ -177,7 +177,7 @@ __global__ void export_f32_kernel(const float *x, const float *y, const float *z
 }  // namespace
 
 namespace pg {
-pg_status alloc_arrays(PsetArrays &A, int pos, int64_t cap, int nvar) {
+pg_status alloc_arrays(PsetArrays &A, int pos, int64_t cap, int nvar, int64_t first) {
   const size_t n = (size_t)std::max<int64_t>(cap, 1);
   // the arrays one after another, each on a 256-byte boundary: sizes first,
   // then addresses
@@ -215,6 +215,18 @@ pg_status alloc_arrays(PsetArrays &A, int pos, int64_t cap, int nvar) {
   }
   base = (char *)A.base;
   layout();
+  if (first < (int64_t)n) {
+    const size_t b = (n - (size_t)first) * 8;
+    cudaError_t z = cudaMemset(A.age + first, 0, b);
+    if (z == cudaSuccess) z = cudaMemset(A.hstep + first, 0, b);
+    // the set's later work may be on a stream that does not wait for this one
+    if (z == cudaSuccess) z = cudaStreamSynchronize(0);
+    if (z != cudaSuccess) {
+      A.free_all();
+      set_error("clearing a particle set's arrays failed: %s", cudaGetErrorString(z));
+      return PG_ERR_CUDA;
+    }
+  }
   return PG_OK;
 }
 
@@ -998,7 +1010,7 @@ pg_status pg_pset_create(pg_fieldset *fs, int64_t n, const double *lon, const do
   ps->fs = fs; ps->pos = pos; ps->seed = seed;
   ps->nvar = fs->ntr;
   PsetArrays A;
-  pg_status r = alloc_arrays(A, pos, n, ps->nvar);
+  pg_status r = alloc_arrays(A, pos, n, ps->nvar, n);
   if (r) { delete ps; return r; }
   set_arrays(ps, A);
   ps->cap = std::max<int64_t>(n, 1);
@@ -1038,7 +1050,7 @@ pg_status pg_pset_add(pg_pset *ps, int64_t n, const double *lon, const double *l
   if (ps->n + n > ps->cap) {
     const int64_t cap = std::max<int64_t>(ps->n + n, ps->cap + ps->cap / 2);
     PsetArrays B;
-    pg_status r = alloc_arrays(B, ps->pos, cap, ps->nvar);
+    pg_status r = alloc_arrays(B, ps->pos, cap, ps->nvar, ps->n + n);
     if (r) return r;
     PsetArrays A = arrays_of(ps);
     const size_t el = pos_elem(ps->pos);
@@ -1654,7 +1666,7 @@ pg_status pg_pset_restore(pg_fieldset *fs, const char *path, pg_pset **out) {
   if (r) return r;
   if (n) {
     PsetArrays B;
-    r = alloc_arrays(B, pos, n, nvar);
+    r = alloc_arrays(B, pos, n, nvar, n);
     if (r) { pg_pset_destroy(ps); return r; }
     const auto arrays = state_arrays(B, pos, nvar, n);
     cudaError_t e = cudaSuccess;

@@ -55,8 +55,12 @@ struct PsetArrays {
   }
 };
 
-// Allocate the arrays of `cap` particles with `nvar` sampled variables.
-pg_status alloc_arrays(PsetArrays &A, int pos, int64_t cap, int nvar);
+// Allocate the arrays of `cap` particles with `nvar` sampled variables.  Ages and
+// step lengths start as zeros from entry `first` on -- the entries that the
+// caller does not write at once -- because a re-sort leaves arrays that no kernel
+// has used where they are, and swaps the two sets: every entry of either has to
+// hold the zero of a new particle by then.
+pg_status alloc_arrays(PsetArrays &A, int pos, int64_t cap, int nvar, int64_t first = 0);
 
 // Arrays of one output slot (device or pinned host), cap rows each.
 struct OutputView {
@@ -168,8 +172,9 @@ struct pg_pset {
   double *var = nullptr;               // [nvar][cap] sampled variables
   double *hstep = nullptr;             // [cap] RKF45 step lengths (0: start from dt)
   int nvar = 0;                        // the field set's scalar fields at creation
-  // whether ages and RKF45 step lengths can be other than the zeros every set
-  // starts with (in both sets of arrays); until then a re-sort leaves them
+  // whether ages and RKF45 step lengths can be other than the zeros that all
+  // entries of both sets of arrays start with (alloc_arrays, new particles);
+  // until then a re-sort leaves them
   bool age_used = false, hstep_used = false;
   double t_min = 0.0, t_max = 0.0;     // range of particle times
   pg_tune tune{256, 0, 0};             // chunk_steps 0: chosen per execute

@@ -316,14 +316,9 @@ cudaError_t prepare_resort(pg_pset *ps) {
   if (ps->alt_cap != ps->cap) {
     ps->alt.free_all();
     ps->alt_cap = 0;
-    if (alloc_arrays(ps->alt, ps->pos, ps->cap, ps->nvar) != PG_OK)
-      return cudaErrorMemoryAllocation;
+    const pg_status r = alloc_arrays(ps->alt, ps->pos, ps->cap, ps->nvar);
+    if (r) return r == PG_ERR_NOMEM ? cudaErrorMemoryAllocation : cudaErrorUnknown;
     ps->alt_cap = ps->cap;
-    // ages and step lengths that no pass has moved yet are zeros in both sets
-    const size_t b = (size_t)std::max<int64_t>(ps->cap, 1) * 8;
-    if ((e = cudaMemset(ps->alt.age, 0, b)) != cudaSuccess) return e;
-    if ((e = cudaMemset(ps->alt.hstep, 0, b)) != cudaSuccess) return e;
-    if ((e = cudaStreamSynchronize(0)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
