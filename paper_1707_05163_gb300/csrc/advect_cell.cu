@@ -35,8 +35,7 @@ cudaError_t launch_advect_cell(const StepArgs &a, int storage, int block, cudaSt
 namespace {
 
 // index coordinate u = (p - x0) / dx in FP64, split into cell and offset
-__device__ __forceinline__ void to_cell(double p, double x0, double d, double rd,
-                                        double sd, int n,
+__device__ __forceinline__ void to_cell(double p, double x0, double d, double rd, int n,
                                         bool periodic, int &i, float &f) {
   if (periodic) {
     double r = p - x0;
@@ -46,7 +45,7 @@ __device__ __forceinline__ void to_cell(double p, double x0, double d, double rd
     }
     p = x0 + r;
   }
-  const double u = quotient(p - x0, d, rd, sd);    // (p - x0) / d
+  const double u = quotient(p - x0, d, rd);    // (p - x0) / d
   double fl = floor(u);
   const double lim = periodic ? (double)(n - 1) : (double)(n - 2);
   if (fl < 0.0) fl = 0.0;
@@ -62,15 +61,15 @@ __device__ __forceinline__ void to_cell(double p, double x0, double d, double rd
 __global__ void to_cell_kernel(GridArgs g, const double *lon, const double *lat,
                                const double *dep, int32_t *ci, int32_t *cj, int32_t *ck,
                                float *fx, float *fy, float *fz, int64_t n) {
-  double rd[3] = {0.0, 0.0, 0.0}, sd[3] = {0.0, 0.0, 0.0};
-  for (int a = 0; a < (g.nz > 1 ? 3 : 2); ++a) reciprocal_for(g.d[a], rd[a], sd[a]);
+  double rd[3] = {0.0, 0.0, 0.0};
+  for (int a = 0; a < (g.nz > 1 ? 3 : 2); ++a) rd[a] = reciprocal_for(g.d[a]);
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
        p += (int64_t)gridDim.x * blockDim.x) {
     int i, j, k = 0;
     float x, y, z = 0.f;
-    to_cell(lon[p], g.x0[0], g.d[0], rd[0], sd[0], g.nx, g.periodic, i, x);
-    to_cell(lat[p], g.x0[1], g.d[1], rd[1], sd[1], g.ny, false, j, y);
-    if (g.nz > 1) to_cell(dep ? dep[p] : g.x0[2], g.x0[2], g.d[2], rd[2], sd[2], g.nz, false, k, z);
+    to_cell(lon[p], g.x0[0], g.d[0], rd[0], g.nx, g.periodic, i, x);
+    to_cell(lat[p], g.x0[1], g.d[1], rd[1], g.ny, false, j, y);
+    if (g.nz > 1) to_cell(dep ? dep[p] : g.x0[2], g.x0[2], g.d[2], rd[2], g.nz, false, k, z);
     ci[p] = i; cj[p] = j; ck[p] = k; fx[p] = x; fy[p] = y; fz[p] = z;
   }
 }

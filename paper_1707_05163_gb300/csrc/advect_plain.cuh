@@ -28,19 +28,20 @@ namespace pg {
 
 // FP64 slow path: locate p, known to lie outside the cached cell of index ci
 // on axis a (n nodes; the last cell is closed when CLOSED): the neighbour
-// where it holds p, else a search.  Refreshes the cell: its index, the
-// reciprocal of its width, and its bounds as order keys.  Returns
+// where it holds p, else a search.  Refreshes the cell: its index, its width
+// w and the width's reciprocal, and its bounds as order keys.  Returns
 // false when p is outside the axis.  The cell found is the largest i <= n-2
 // with x[i] <= p.
-__device__ __forceinline__ void set_cell64(double lo, double hi, bool closed, double &r, double &s,
+__device__ __forceinline__ void set_cell64(double lo, double hi, bool closed, double &r, double &w,
                                            long long &klo, long long &khi) {
-  reciprocal_for(hi - lo, r, s);
+  w = hi - lo;
+  r = reciprocal_for(w);
   klo = order_key(lo);
   khi = order_key(hi) + (closed ? 1 : 0);
 }
 template <bool CLOSED>
 __device__ __forceinline__ bool relocate64(const GridArgs &g, int a, int n, double p, int &ci,
-                                           double &r, double &s, long long &klo, long long &khi) {
+                                           double &r, double &w, long long &klo, long long &khi) {
   const double *x = axis<double>(g, a);
   int i = -1;
   double lo = 0.0, hi = 0.0;
@@ -61,7 +62,7 @@ __device__ __forceinline__ bool relocate64(const GridArgs &g, int a, int n, doub
     lo = x[i]; hi = x[i + 1];
   }
   ci = i;
-  set_cell64(lo, hi, CLOSED && i == n - 2, r, s, klo, khi);
+  set_cell64(lo, hi, CLOSED && i == n - 2, r, w, klo, khi);
   return true;
 }
 
@@ -239,22 +240,22 @@ __device__ __forceinline__ int velocity(const A &a, Sampler<Real, Store, NF, D3,
         if (is_per<GEO>(g)) {
           if (q >= axis_hi(g, 0, q)) {          // the wrap cell
             c.ci = g.nx - 1;
-            set_cell64(axis_hi(g, 0, q), lon_end(g, q), false, c.rx, c.sx, c.klo[0], c.khi[0]);
-          } else if (!relocate64<false>(g, 0, g.nx, q, c.ci, c.rx, c.sx, c.klo[0], c.khi[0])) {
+            set_cell64(axis_hi(g, 0, q), lon_end(g, q), false, c.rx, c.wx, c.klo[0], c.khi[0]);
+          } else if (!relocate64<false>(g, 0, g.nx, q, c.ci, c.rx, c.wx, c.klo[0], c.khi[0])) {
             return 1;
           }
-        } else if (!relocate64<true>(g, 0, g.nx, q, c.ci, c.rx, c.sx, c.klo[0], c.khi[0])) {
+        } else if (!relocate64<true>(g, 0, g.nx, q, c.ci, c.rx, c.wx, c.klo[0], c.khi[0])) {
           return 1;
         }
         c.dirty |= 1;
       }
       if (!hy) {
-        if (!relocate64<true>(g, 1, g.ny, lat, c.cj, c.ry, c.sy, c.klo[1], c.khi[1])) return 1;
+        if (!relocate64<true>(g, 1, g.ny, lat, c.cj, c.ry, c.wy, c.klo[1], c.khi[1])) return 1;
         c.dirty |= 1;
       }
       if constexpr (D3) {
         if (!hz) {
-          if (!relocate64<true>(g, 2, g.nz, dep, c.ck, c.rz, c.sz, c.klo[2], c.khi[2])) return 2;
+          if (!relocate64<true>(g, 2, g.nz, dep, c.ck, c.rz, c.wz, c.klo[2], c.khi[2])) return 2;
           c.dirty |= 1;
         }
       } else {
@@ -264,14 +265,14 @@ __device__ __forceinline__ int velocity(const A &a, Sampler<Real, Store, NF, D3,
     const double xlo = from_order_key(c.klo[0]), ylo = from_order_key(c.klo[1]);
     const double zlo = D3 ? from_order_key(c.klo[2]) : 0.0;
     const double ax = q - xlo, ay = lat - ylo, az = D3 ? dep - zlo : 0.0;
-    double xi = times_reciprocal(ax, c.rx, c.sx), eta = times_reciprocal(ay, c.ry, c.sy);
-    double zeta = D3 ? times_reciprocal(az, c.rz, c.sz) : 0.0;
+    double xi = fit_quotient(ax, c.wx, c.rx), eta = fit_quotient(ay, c.wy, c.ry);
+    double zeta = D3 ? fit_quotient(az, c.wz, c.rz) : 0.0;
     bool fit = fraction_fit(ax, c.rx) & fraction_fit(ay, c.ry);
     if constexpr (D3) fit = fit & fraction_fit(az, c.rz);
     if (!fit) {
-      xi = ax / ((c.ci == g.nx - 1 ? lon_end(g, q) : g.lon[c.ci + 1]) - g.lon[c.ci]);
-      eta = ay / (g.lat[c.cj + 1] - g.lat[c.cj]);
-      if constexpr (D3) zeta = az / (g.depth[c.ck + 1] - g.depth[c.ck]);
+      xi = ax / c.wx;
+      eta = ay / c.wy;
+      if constexpr (D3) zeta = az / c.wz;
     }
     const int r = sample_fields(a, c, ck, off, xi, eta, zeta, vel);
     if (r) return r;
