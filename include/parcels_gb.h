@@ -153,8 +153,11 @@ typedef struct {
                         /* fewer in a launch that would leave multiprocessors idle)  */
     int resort_steps;   /* Morton re-sort before the first launch of an execute and
                            every this many steps (0: never)                          */
-    int chunk_steps;    /* at most this many steps per kernel launch (0: chosen by   */
-                        /* the library; results do not depend on it)                 */
+    int chunk_steps;    /* at most this many steps per kernel launch (0: up to 1440  */
+                        /* where no result depends on it -- FP64 positions; snapshot */
+                        /* times, and of fixed steps all times, in whole seconds --  */
+                        /* else 64; elsewhere two lengths may round a time           */
+                        /* differently)                                              */
 } pg_tune;
 
 /* Snapshot source for streamed fields (the counterpart of advancing the

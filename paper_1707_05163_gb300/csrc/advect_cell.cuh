@@ -109,6 +109,7 @@ __device__ __forceinline__ int step_cell(const StepArgs &a, Sampler<float, Store
   const float half = 0.5f * h;
   const int nst = a.k.scheme == 0 ? 1 : 4;
   int r;
+  start_step32(c, ck);
   acc[0] = 0.f; acc[1] = 0.f; acc[2] = 0.f;
 #pragma unroll 1
   for (int q = 0; q < nst; ++q) {

@@ -276,6 +276,8 @@ struct Sampler {
     if constexpr (sizeof(Real) == 8) {
       for (int a = 0; a < 3; ++a) { klo[a] = 1; khi[a] = 0; }
       ta = tb = rt = 0.0;
+    } else {
+      span = 0.f;
     }
   }
 };
@@ -481,6 +483,14 @@ __device__ __forceinline__ float kh_of(const KernArgs &k, float) { return k.kh_f
 __device__ __forceinline__ double w_of(const KernArgs &k, double) { return k.w_sink; }
 __device__ __forceinline__ float w_of(const KernArgs &k, float) { return k.w_sink_f; }
 
+// FP32, once per step: a step that starts on the cached interval's last snapshot
+// belongs to the next interval (its other stages may end on the last one), so
+// the cached interval holds none of its times and the first stage moves on.
+template <typename Store, int NF, bool D3, int GEO>
+__device__ __forceinline__ void start_step32(Sampler<float, Store, NF, D3, GEO> &c, const Clock &ck) {
+  if (!(ck.d < c.span)) c.span = -1.f;
+}
+
 // FP32: bring the snapshot interval of the stage time (step start + off)
 // and the corner cache up to date -- the slow part of a stage, skipped while
 // the stage stays in the cached cell and interval.  The stage time is an
@@ -530,9 +540,8 @@ __device__ __forceinline__ float tau32(const A &a, const Sampler<float, Store, N
 // weights formed once per stage (bilinear, or trilinear as the bilinear
 // weights times 1 - zeta and zeta).  The sum runs in corner order (i, j),
 // (i+1, j), (i, j+1), (i+1, j+1)[, the same on level k+1] as one chain of
-// fused multiply-adds; on a cell face the weights of the far corners are
-// exactly 0 and the remaining terms come in the same order from either
-// neighbouring cell, so the two cells give the same value there.
+// fused multiply-adds; on a cell's lower face the weights of the far corners
+// are exactly 0.
 template <int NC>
 __device__ __forceinline__ void corner_weights(float xi, float eta, float zeta, float (&w)[NC]) {
   const float x0 = 1.f - xi, y0 = 1.f - eta;
@@ -572,9 +581,7 @@ __device__ __forceinline__ int nearest_corner(Real xi, Real eta, Real zeta) {
 }
 
 // FP32 field values from the cached corners: spatial interpolation in both
-// snapshots (weighted_sum), then (1 - tau) a + tau b, exact at both ends, so a stage time on
-// a snapshot gives the same value from either neighbouring interval (results
-// do not depend on which interval a thread has cached).  A steady field holds
+// snapshots (weighted_sum), then (1 - tau) a + tau b, exact at both ends.  A steady field holds
 // its snapshot in both slots with tau = 0, which returns a exactly, so there
 // is no branch on steadiness.  One NaN test per stage covers all components
 // (same outcome as a test per value: PG_NAN, state untouched) and leaves the

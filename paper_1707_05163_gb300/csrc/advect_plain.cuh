@@ -15,9 +15,14 @@
 //     out the oracle's operations in the oracle's order, including the FP64
 //     time interpolation of every stage and its cell and interval tie-breaks;
 //   Real = float: the FP32 path, where stage times are FP32 offsets inside
-//     the cached snapshot interval, cell and interval bounds are inclusive on
-//     both sides (continuity makes the two choices at a shared node equal),
-//     and no FP64 arithmetic runs per stage.
+//     the cached snapshot interval and no FP64 arithmetic runs per stage.
+// Either way a position on a node belongs to the cell above it, as in the
+// definition, the last node of a closed axis aside, and a step that starts on a
+// snapshot to the interval after it (in FP32 its later stages may end on the
+// last snapshot of their interval): what a step computes depends on its position
+// and time alone and not on the cell and interval that the particle came from.
+// (The two choices are not equal in FP32: (hi - lo) RN(1 / (hi - lo)) is 1 -
+// 2^-24 for some widths, 41 or seven hours in seconds among them.)
 #pragma once
 
 #include <type_traits>
@@ -66,8 +71,9 @@ __device__ __forceinline__ bool relocate64(const GridArgs &g, int a, int n, doub
   return true;
 }
 
-// FP32 slow path: locate p, known to lie outside the cached cell [lo, hi] of
-// index ci on axis a (n nodes), and refresh the cell.  A move to a neighbour
+// FP32 slow path: locate p, known to lie outside the cached cell [lo, hi) of
+// index ci on axis a (n nodes), and refresh the cell; `top` is the bound of the
+// last cell, the float above its node where the axis ends there.  A move to a neighbour
 // cell costs one node (the far node of the neighbour; the shared node is the
 // old lo or hi); anything else searches the axis.  The cell found is the
 // largest i <= n-2 with x[i] <= p, as a fresh search gives.  SELECT: both
@@ -76,8 +82,8 @@ __device__ __forceinline__ bool relocate64(const GridArgs &g, int a, int n, doub
 // spills) and slower in the 2-D ones, which keep the branches; the cell
 // found is the same either way.
 template <bool SELECT>
-__device__ __forceinline__ void relocate32(const GridArgs &g, int a, int n, float p, int &ci,
-                                           float &lo, float &hi, float &rinv) {
+__device__ __forceinline__ void relocate32(const GridArgs &g, int a, int n, float p, float top,
+                                           int &ci, float &lo, float &hi, float &rinv) {
   const float *x = axis<float>(g, a);
   if constexpr (SELECT) {
     const int cm = ci - 1 < 0 ? 0 : ci - 1;
@@ -86,18 +92,19 @@ __device__ __forceinline__ void relocate32(const GridArgs &g, int a, int n, floa
     const bool held = (ci >= 0) & (ci <= n - 2);
     const bool below = p < lo;
     const bool down = held & below & (ci >= 1) & (xm <= p);
-    const bool up =
-        held & !below & (ci + 1 <= n - 2) & ((p < x2) | ((ci + 1 == n - 2) & (p == x2)));
+    const bool up = held & !below & (ci + 1 < n - 2) & (p < x2);
     int i = down ? ci - 1 : ci + 1;
     float nlo = down ? xm : hi, nhi = down ? lo : x2;
+    float end = nhi;
     if (!(down | up)) {
       i = axis_search<float>(g, a, n, p);
       nlo = x[i];
       nhi = x[i + 1];
+      end = i == n - 2 ? top : nhi;
     }
     ci = i;
     lo = nlo;
-    hi = nhi;
+    hi = end;
     rinv = __frcp_rn(nhi - nlo);
     return;
   }
@@ -109,19 +116,21 @@ __device__ __forceinline__ void relocate32(const GridArgs &g, int a, int n, floa
         const float xm = x[ci - 1];
         if (xm <= p) { i = ci - 1; nlo = xm; nhi = lo; }
       }
-    } else if (ci + 1 <= n - 2) {   // p > hi
+    } else if (ci + 1 < n - 2) {   // p >= hi
       const float x2 = x[ci + 2];
-      if (p < x2 || (ci + 1 == n - 2 && p == x2)) { i = ci + 1; nlo = hi; nhi = x2; }
+      if (p < x2) { i = ci + 1; nlo = hi; nhi = x2; }
     }
   }
+  float end = nhi;
   if (i < 0) {
     i = axis_search<float>(g, a, n, p);
     nlo = x[i];
     nhi = x[i + 1];
+    end = i == n - 2 ? top : nhi;
   }
   ci = i;
   lo = nlo;
-  hi = nhi;
+  hi = end;
   rinv = __frcp_rn(nhi - nlo);   // correctly rounded, as 1.0f / (hi - lo)
 }
 
@@ -132,8 +141,9 @@ __device__ __forceinline__ void relocate32(const GridArgs &g, int a, int n, floa
 // the interval; later stages of the step then take it too, at no cost in
 // results.
 template <typename Real, typename Store, int NF, bool D3, int GEO, class A>
-__device__ __forceinline__ void step_in_interval(const A &a, const Sampler<Real, Store, NF, D3, GEO> &c,
+__device__ __forceinline__ void step_in_interval(const A &a, Sampler<Real, Store, NF, D3, GEO> &c,
                                                  Clock &ck, float h) {
+  start_step32(c, ck);
   const float de = ck.d + h;
   ck.tin = (a.f.nt == 1) | ((c.s0 >= 0) & (fminf(ck.d, de) >= 0.f) & (fmaxf(ck.d, de) <= c.span));
 }
@@ -155,8 +165,8 @@ __device__ __forceinline__ int velocity(const A &a, Sampler<Real, Store, NF, D3,
     // the zonal seam misses and the slow path reduces it.
     const float x0 = axis_lo(g, 0, lon);
     float q = lon;
-    bool hit = (q >= c.xlo) & (q <= c.xhi) & (lat >= c.ylo) & (lat <= c.yhi);
-    if constexpr (D3) hit = hit & (dep >= c.zlo) & (dep <= c.zhi);
+    bool hit = (q >= c.xlo) & (q < c.xhi) & (lat >= c.ylo) & (lat < c.yhi);
+    if constexpr (D3) hit = hit & (dep >= c.zlo) & (dep < c.zhi);
     hit = hit & ck.tin;
     float xi, eta, zeta = 0.f;
     if (!hit) {
@@ -168,7 +178,7 @@ __device__ __forceinline__ int velocity(const A &a, Sampler<Real, Store, NF, D3,
       // each axis whose cached cell fails is located again (the Sampler
       // starts with empty cells on every axis, so all fail the first time)
       const int nan = (!(lon == lon) | !(lat == lat) | !(dep == dep)) ? 3 : 0;
-      if (!((q >= c.xlo) & (q <= c.xhi))) {
+      if (!((q >= c.xlo) & (q < c.xhi))) {
         if (is_per<GEO>(g)) {
           if (!isfinite(lon)) return nan ? nan : 1;
           if (!(q >= x0 && q < x0 + 360.0f)) q = wrap_lon(lon, x0);
@@ -182,19 +192,19 @@ __device__ __forceinline__ int velocity(const A &a, Sampler<Real, Store, NF, D3,
           c.xhi = lon_end(g, q);
           c.rx = __frcp_rn(c.xhi - c.xlo);
         } else {
-          relocate32<D3>(g, 0, g.nx, q, c.ci, c.xlo, c.xhi, c.rx);
+          relocate32<D3>(g, 0, g.nx, q, is_per<GEO>(g) ? axis_hi(g, 0, q) : g.topf[0], c.ci, c.xlo, c.xhi, c.rx);
         }
       }
-      if (!((lat >= c.ylo) & (lat <= c.yhi))) {
+      if (!((lat >= c.ylo) & (lat < c.yhi))) {
         if (!(lat >= axis_lo(g, 1, lat) && lat <= axis_hi(g, 1, lat))) return nan ? nan : 1;
         c.dirty |= 1;
-        relocate32<D3>(g, 1, g.ny, lat, c.cj, c.ylo, c.yhi, c.ry);
+        relocate32<D3>(g, 1, g.ny, lat, g.topf[1], c.cj, c.ylo, c.yhi, c.ry);
       }
       if constexpr (D3) {
-        if (!((dep >= c.zlo) & (dep <= c.zhi))) {
+        if (!((dep >= c.zlo) & (dep < c.zhi))) {
           if (!(dep >= axis_lo(g, 2, dep) && dep <= axis_hi(g, 2, dep))) return nan ? nan : 2;
           c.dirty |= 1;
-          relocate32<D3>(g, 2, g.nz, dep, c.ck, c.zlo, c.zhi, c.rz);
+          relocate32<D3>(g, 2, g.nz, dep, g.topf[2], c.ck, c.zlo, c.zhi, c.rz);
         }
       } else {
         c.ck = 0;
@@ -536,7 +546,11 @@ __device__ __forceinline__ unsigned long long rkf45_steps(
     if (sgn * (target - t) < sgn * h) { h = target - t; clipped = true; }
     ck.t = t;
     if constexpr (sizeof(Real) == 4) {
-      ck.d = c.s0 >= 0 ? (float)(t - c.ta) : 0.f;
+      // a trial may have moved the cached interval past the step's start: an
+      // offset outside it (below zero) makes the first stage find the start's own,
+      // as the first step of a launch does
+      ck.d = (float)(t - c.ta);
+      if (!((c.s0 >= 0) & (ck.d >= 0.f) & (ck.d < c.span))) ck.d = -1.f;
       step_in_interval(a, c, ck, (float)h);
     }
     Real x4[3], err;

@@ -274,6 +274,7 @@ GridArgs grid_args(const pg_fieldset *fs) {
     const std::vector<double> &x = a == 0 ? fs->lon : (a == 1 ? fs->lat : fs->depth);
     g.lo[a] = x.front(); g.hi[a] = x.back();
     g.lof[a] = (float)x.front(); g.hif[a] = (float)x.back();
+    g.topf[a] = std::nextafter(g.hif[a], std::numeric_limits<float>::infinity());
   }
   const double D = 1852.0 * 60.0;
   for (int a = 0; a < 3; ++a) {
@@ -1285,22 +1286,27 @@ pg_status pg_execute_records(pg_pset *ps, const pg_kernel *k, double runtime, do
 // location and corner gather of each particle, and a small set is at rest
 // between launches, so launches are long (1440 steps; 38 launches of 64 took
 // 100 particles 2.7 ms for 2400 steps) -- but only where their length cannot
-// show in the results: the FP32 forms count a launch's steps from its start
-// time, and keep a step's time as an FP32 offset in its snapshot interval,
-// advanced step by step and formed anew at each launch, which is exact while
-// times, steps and interval are whole seconds below 2^24.  Anything else
-// keeps 64.
-static int default_chunk(const pg_pset *ps, const pg_kernel *k, double dt) {
+// show in the results: the FP32 forms keep a stage's time as an FP32 offset in
+// its snapshot interval, and find the interval's start from the first stage time
+// in it.  RKF45, whose steps have any length, forms the offset anew at each
+// step: exact while the snapshot times and the period are whole seconds and no
+// time lies before the first snapshot or zero.  Fixed steps advance it step by
+// step from their launch's start time: exact while all times are whole seconds
+// and it stays below 2^24.  Anything else keeps 64.
+static int default_chunk(const pg_pset *ps, const pg_kernel *k, double dt, double t_end) {
   const pg_fieldset *fs = ps->fs;
   constexpr int kLong = 1440, kShort = 64;
-  if (ps->pos == PG_POS_F64 || k->scheme == PG_RKF45) return kLong;
+  if (ps->pos == PG_POS_F64) return kLong;
   auto whole = [](double v) { return std::fabs(v) < 9.0e15 && v == std::floor(v); };
-  if (!whole(dt) || ps->t_min != ps->t_max || !whole(ps->t_min) || !whole(fs->period)) return kShort;
+  if (!whole(fs->period)) return kShort;
   double gap = fs->period > 0.0 ? fs->times[0] + fs->period - fs->times.back() : 0.0;
   for (int s = 0; s < fs->nt; ++s) {
     if (!whole(fs->times[s])) return kShort;
     if (s > 0) gap = std::max(gap, fs->times[s] - fs->times[s - 1]);
   }
+  if (k->scheme == PG_RKF45)
+    return fs->times[0] >= 0.0 && (dt > 0.0 ? ps->t_min : t_end) >= fs->times[0] ? kLong : kShort;
+  if (!whole(dt) || ps->t_min != ps->t_max || !whole(ps->t_min)) return kShort;
   return gap + std::fabs(dt) < 16777216.0 ? kLong : kShort;
 }
 
@@ -1419,7 +1425,7 @@ static pg_status execute_loop(pg_pset *ps, const pg_kernel *k, double runtime, d
   CU(cudaMemsetAsync(ps->d_counter, 0, 16, st));     // the error word with it
 
   const double chunk_len =
-      std::fabs(dt) * (ps->tune.chunk_steps > 0 ? ps->tune.chunk_steps : default_chunk(ps, k, dt));
+      std::fabs(dt) * (ps->tune.chunk_steps > 0 ? ps->tune.chunk_steps : default_chunk(ps, k, dt, t_end));
   const double resort_len = ps->tune.resort_steps > 0 ? std::fabs(dt) * ps->tune.resort_steps : 0.0;
   double next_out = output_dt > 0.0 ? t_begin + sgn * output_dt : t_end;
   double next_sort = resort_len > 0.0 ? t_begin + sgn * resort_len : t_end;

@@ -30,6 +30,7 @@ struct GridArgs {
   float lon_end_f;
   double lo[3], hi[3];       // first and last node of each axis (kernel
   float lof[3], hif[3];      // parameters, so range tests load nothing)
+  float topf[3];             // the float above hif: bound of a last cell [lo, hi]
   // uniform axes, cell form: spacing, and metres -> cells factors (lon on a
   // sphere: 1 / (D dlon), still to be divided by cos(lat))
   double d[3];
