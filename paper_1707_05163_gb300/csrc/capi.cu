@@ -138,7 +138,8 @@ bool kernel_ptr(const void *p, int device) {
 }
 
 // New particles [0, n) of the given arrays (already offset): positions from
-// FP64 sources (x, y; z may be null: zfill) unless the set is in the cell form
+// FP64 sources (x, y; z may be null: zfill; an FP64 set's own array: already
+// there) unless the set is in the cell form
 // (to_cell_kernel), the start time, consecutive ids, and the zero or NaN
 // start of everything else -- one pass instead of a launch per array.
 template <typename Real>
@@ -918,47 +919,74 @@ pg_status pg_kernel_destroy(pg_kernel *k) {
   return PG_OK;
 }
 
+// A staging buffer on the device for `arrays` arrays of doubles of a set's n
+// entries: whole, or, where the memory is not there (24 bytes per particle are
+// half an FP32 set's own state), of fewer rows, which the caller works through
+// piece by piece -- down to 64K rows, and to the size of one array.
+static cudaError_t alloc_staging(double **tmp, int arrays, int64_t n, int64_t &rows) {
+  constexpr int64_t kMinRows = 65536;
+  rows = n;
+  *tmp = nullptr;
+  if (arrays == 0) return cudaSuccess;
+  for (;;) {
+    const cudaError_t e = dev_alloc((void **)tmp, (size_t)rows * 8 * arrays);
+    if (e != cudaErrorMemoryAllocation || (rows <= kMinRows && rows * arrays <= n)) return e;
+    if (rows == 1) return e;
+    cudaGetLastError();
+    rows = (rows + 1) / 2;
+  }
+}
+
 static pg_status fill_particles(pg_pset *ps, int64_t off, int64_t n, const double *lon,
                                 const double *lat, const double *depth, const double *time,
                                 double t0, const uint64_t *ids, uint64_t id_base,
                                 cudaStream_t st, double &tmin, double &tmax) {
   const pg_fieldset *fs = ps->fs;
   const int sm = fs->sm_count;
-  const bool cell = ps->pos == PG_POS_CELL;
+  const bool cell = ps->pos == PG_POS_CELL, f64 = ps->pos == PG_POS_F64;
   // sources a kernel can read stay where they are; the others are copied to
-  // the device (at the copy engines' rate from pinned memory) and rounded or
-  // split there
+  // the device (at the copy engines' rate from pinned memory), FP64 positions
+  // into place and the others' to be rounded or split there
   const double *src[3] = {lon, lat, depth};
+  bool via[3];
   int staged = 0;
-  for (const double *p : src) staged += p && !kernel_ptr(p, fs->device);
+  for (int q = 0; q < 3; ++q) staged += via[q] = src[q] && !kernel_ptr(src[q], fs->device);
   double *tmp = nullptr;
-  if (staged) CU(dev_alloc((void **)&tmp, (size_t)n * 8 * staged));
+  int64_t piece = n;
+  CU(alloc_staging(&tmp, f64 ? 0 : staged, n, piece));
   cudaError_t e = cudaSuccess;
-  double *next = tmp;
-  for (const double *&p : src)
-    if (p && !kernel_ptr(p, fs->device)) {
-      if (e == cudaSuccess) e = cudaMemcpyAsync(next, p, n * 8, cudaMemcpyDefault, st);
-      p = next;
-      next += n;
-    }
-  PsetArrays A = arrays_of(ps);
   const size_t el = pos_elem(ps->pos);
-  if (cell) {
-    if (e == cudaSuccess)
-      e = launch_to_cell(grid_args(fs), src[0], src[1], src[2], ps->ci + off, ps->cj + off,
-                         ps->ck + off, ps->fx + off, ps->fy + off, ps->fz + off, n, sm, st);
-    src[0] = nullptr;
-  } else {
-    A.x = (char *)A.x + off * el; A.y = (char *)A.y + off * el; A.z = (char *)A.z + off * el;
-  }
-  A.time += off; A.id += off; A.step += off; A.status += off; A.age += off; A.hstep += off;
-  if (A.var) A.var += off;
-  if (e == cudaSuccess) {
-    auto kern = ps->pos == PG_POS_F64 ? init_particles_kernel<double> : init_particles_kernel<float>;
-    kern<<<grid_for(n, sm), 256, 0, st>>>(src[0], src[1], src[2], 0.0, A, n, time == nullptr, t0,
-                                          ids == nullptr, id_base, ps->nvar, ps->cap);
-    note_launches(1);
-    e = cudaGetLastError();
+  for (int64_t p = 0; p < n && e == cudaSuccess; p += piece) {
+    const int64_t m = std::min(piece, n - p), at = off + p;
+    PsetArrays A = arrays_of(ps);
+    void *const place[3] = {A.x, A.y, A.z};
+    const double *from[3];
+    double *next = tmp;
+    for (int q = 0; q < 3; ++q) {
+      from[q] = src[q] ? src[q] + p : nullptr;
+      if (!via[q]) continue;
+      double *to = f64 ? (double *)place[q] + at : next;
+      if (e == cudaSuccess) e = cudaMemcpyAsync(to, from[q], m * 8, cudaMemcpyDefault, st);
+      from[q] = to;
+      next += f64 ? 0 : m;
+    }
+    if (cell) {
+      if (e == cudaSuccess)
+        e = launch_to_cell(grid_args(fs), from[0], from[1], from[2], A.ci + at, A.cj + at, A.ck + at,
+                           A.fx + at, A.fy + at, A.fz + at, m, sm, st);
+      from[0] = nullptr;
+    } else {
+      A.x = (char *)A.x + at * el; A.y = (char *)A.y + at * el; A.z = (char *)A.z + at * el;
+    }
+    A.time += at; A.id += at; A.step += at; A.status += at; A.age += at; A.hstep += at;
+    if (A.var) A.var += at;
+    if (e == cudaSuccess) {
+      auto kern = f64 ? init_particles_kernel<double> : init_particles_kernel<float>;
+      kern<<<grid_for(m, sm), 256, 0, st>>>(from[0], from[1], from[2], 0.0, A, m, time == nullptr, t0,
+                                            ids == nullptr, id_base + (uint64_t)p, ps->nvar, ps->cap);
+      note_launches(1);
+      e = cudaGetLastError();
+    }
   }
   tmin = t0; tmax = t0;
   std::vector<double> h;
@@ -1121,30 +1149,33 @@ pg_status pg_pset_get(const pg_pset *ps, double *lon, double *lat, double *depth
   } else if (lon || lat || depth) {
     // converted straight into destinations a kernel can write; through a
     // buffer on the device into the others
-    double *dst[3] = {lon, lat, depth}, *out[3] = {lon, lat, depth};
+    double *dst[3] = {lon, lat, depth};
     int staged = 0;
     bool via[3];
-    for (int q = 0; q < 3; ++q) {
-      via[q] = dst[q] && !kernel_ptr(dst[q], ps->fs->device);
-      staged += via[q];
+    for (int q = 0; q < 3; ++q) staged += via[q] = dst[q] && !kernel_ptr(dst[q], ps->fs->device);
+    int64_t piece = n;
+    CU(alloc_staging(&tmp, staged, n, piece));
+    cudaError_t e = cudaSuccess;
+    for (int64_t p = 0; p < n && e == cudaSuccess; p += piece) {
+      const int64_t m = std::min(piece, n - p);
+      double *out[3], *next = tmp;
+      for (int q = 0; q < 3; ++q) {
+        out[q] = via[q] ? next : (dst[q] ? dst[q] + p : nullptr);
+        if (via[q]) next += m;
+      }
+      if (ps->pos == PG_POS_CELL) {
+        e = launch_from_cell(grid_args(ps->fs), ps->ci + p, ps->cj + p, ps->ck + p, ps->fx + p,
+                             ps->fy + p, ps->fz + p, out[0], out[1], out[2], m, ps->fs->sm_count, st);
+      } else {
+        export_f32_kernel<<<grid_for(m, ps->fs->sm_count), 256, 0, st>>>(
+            (const float *)ps->x + p, (const float *)ps->y + p, (const float *)ps->z + p, out[0],
+            out[1], out[2], m);
+        note_launches(1);
+        e = cudaGetLastError();
+      }
+      for (int q = 0; q < 3 && e == cudaSuccess; ++q)
+        if (via[q]) e = cudaMemcpyAsync(dst[q] + p, out[q], m * 8, cudaMemcpyDefault, st);
     }
-    if (staged) CU(dev_alloc((void **)&tmp, (size_t)n * 8 * staged));
-    double *next = tmp;
-    for (int q = 0; q < 3; ++q)
-      if (via[q]) { out[q] = next; next += n; }
-    cudaError_t e;
-    if (ps->pos == PG_POS_CELL) {
-      e = launch_from_cell(grid_args(ps->fs), ps->ci, ps->cj, ps->ck, ps->fx, ps->fy, ps->fz,
-                           out[0], out[1], out[2], n, ps->fs->sm_count, st);
-    } else {
-      export_f32_kernel<<<grid_for(n, ps->fs->sm_count), 256, 0, st>>>(
-          (const float *)ps->x, (const float *)ps->y, (const float *)ps->z, out[0], out[1], out[2],
-          n);
-      note_launches(1);
-      e = cudaGetLastError();
-    }
-    for (int q = 0; q < 3 && e == cudaSuccess; ++q)
-      if (via[q]) e = cudaMemcpyAsync(dst[q], out[q], n * 8, cudaMemcpyDefault, st);
     if (e != cudaSuccess) {
       set_error("copy failed: %s", cudaGetErrorString(e));
       r = PG_ERR_CUDA;
