@@ -589,10 +589,10 @@ cudaError_t backward(pg_mlp *n, int64_t rows, cudaStream_t st) {
     if (is_tc(l)) {
       // dPre of layer l-1 = (dPre W) * GELU'(pre) in one product (B = W^T
       // [din x dout]), each element over the pre-activation it was formed
-      // with, with its column sums; in FP32 only for a next layer that goes
-      // the other way
+      // with, and the column sums of its FP32 values: all that the next layer
+      // reads, on either engine
       if ((e = gemm_nt_tc(dcur, dout, n->wbt + n->woff[l], dout, rows, din, dout, nullptr, 2,
-                          is_tc(l - 1) ? nullptr : n->dy, dprev, nullptr, din, st, n->d_err, dprev,
+                          nullptr, dprev, nullptr, din, st, n->d_err, dprev,
                           n->colpart + (size_t)(l - 1) * n->col_rows * wmax, &nparts)) != cudaSuccess)
         return e;
       have_part = true;
