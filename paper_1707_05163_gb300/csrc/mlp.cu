@@ -1,13 +1,14 @@
 // mlp.cu -- the flow-map surrogate's MLP on BF16 tensor cores with FP32
 // accumulation: forward (inference and training), backward, Adam.
 //
-// Network: n_in -> width -> ... (depth hidden layers, GELU) -> n_out.  All
+// Network: n_in -> width -> ... (depth hidden layers, GELU) -> n_out.  The
 // matrix products are one kernel shape, C[M x N] = A[M x K] . B[N x K]^T with
-// both operands K-contiguous BF16 and an FP32 accumulator; the other
-// products of back-propagation reach that shape through explicit transposes:
+// both operands K-contiguous BF16 and an FP32 accumulator:
 //   forward   Y  = X  W^T      A = X [M x in],      B = W  [out x in]
 //   input grad dX = dY W       A = dY [M x out],    B = W^T [in x out]
 //   weight grad dW = dY^T X    A = dY^T [out x M],  B = X^T [in x M]
+// the last through transposed copies on mma.sync; on tcgen05 it reads the
+// row-major matrices as they are (gemm_tn_splitk_tc).
 // Widths are padded to multiples of 64 (inputs and outputs zero-padded), so
 // every tile is full in N and K; M may be ragged.
 //
@@ -216,8 +217,8 @@ __global__ void transpose_bf16(const __nv_bfloat16 *in, int rows, int cols, int 
   }
 }
 
-// dPre = dAct * gelu'(pre), both [M x N] (dAct FP32 in, dPre BF16 out), and
-// bias gradient partials (column sums) in FP32.
+// dPre = dAct * gelu'(pre), both [M x N]: dAct FP32 in, dPre BF16 out and, for
+// the bias gradient's column sums, in FP32.
 __global__ void gelu_backward(const float *dact, const __nv_bfloat16 *pre, int64_t M, int N,
                               __nv_bfloat16 *dpre, float *dpre_f32) {
   const int64_t total = M * N;

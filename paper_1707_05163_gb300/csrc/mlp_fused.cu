@@ -45,8 +45,10 @@
 // clocks per tile, 1M rows in 445 us; what is left is the epilogue's latency
 // of each layer, about 4k clocks of a tile.  Each tile has its own accumulator and its own
 // 128 x 256 BF16 activation buffer; a CTA left with one tile alternates the
-// accumulators instead.  The next layer's first four K-pieces need only the
-// first half of the activations and start while the second half is written.
+// accumulators instead.  The first two of a layer's four K-pieces need only the
+// first half of the activations: of a tile alone they start when that is
+// written; of a pair, whose accumulator they overwrite, once it has been read,
+// with each warp's last 32 columns still to be written.
 // An activation half is overwritten only after every product that reads it
 // has completed (the commit that makes an accumulator ready covers all
 // earlier products).

@@ -184,10 +184,11 @@ __global__ void scatter_kernel(const uint32_t *key, uint32_t *offset, uint32_t *
 
 // Arrays of a set's state moved in one pass: entry p of dst from entry perm[p]
 // of src (perm null: entry p).  A permuted pass is bound by its scattered
-// reads, so arrays share a pass only while they stay in L2 together: the
-// passes of a set of up to a million particles take them all (one launch in
-// place of twelve); of 10M particles, all at once were 1.03 ms, and passes
-// of at most kPassBytes 0.5 ms.
+// reads, so arrays share a pass only while they stay in L2 together (129 MB on
+// the chip this library is compiled for, source and destination): the passes of
+// a set of up to a million particles take them all (one launch in place of
+// twelve); of 10M particles, all at once were 1.03 ms, and passes of at most
+// kPassBytes 0.39 ms.
 constexpr int kPassArrays = 8;
 constexpr size_t kPassBytes = (size_t)48 << 20;
 struct StatePass {
