@@ -1039,7 +1039,8 @@ pg_status pg_pset_create(pg_fieldset *fs, int64_t n, const double *lon, const do
   ps->fs = fs; ps->pos = pos; ps->seed = seed;
   ps->nvar = fs->ntr;
   PsetArrays A;
-  pg_status r = alloc_arrays(A, pos, n, ps->nvar, n);
+  // (the one entry of an empty set is written by its first add)
+  pg_status r = alloc_arrays(A, pos, n, ps->nvar, std::max<int64_t>(n, 1));
   if (r) { delete ps; return r; }
   set_arrays(ps, A);
   ps->cap = std::max<int64_t>(n, 1);

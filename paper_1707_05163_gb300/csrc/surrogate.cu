@@ -374,10 +374,13 @@ pg_status pg_surrogate_run(pg_pset *ps, pg_mlp *net, const pg_kernel *k, int nst
     cleanup();
     return r;
   }
+  // their ages and RKF45 step lengths start from zero where the kernel uses
+  // them (always clearing them took some 50 us of a run of 1.7 ms)
+  const bool uses = (k->beh & PG_AGE) || k->scheme == PG_RKF45;
   auto copy_set = [&](pg_pset *dst, const pg_pset *src) -> cudaError_t {
-    if (dst->cap < src->n) {
+    if (dst->cap < src->n || (uses && dst->n == 0 && src->n > 0)) {
       PsetArrays A;
-      if (alloc_arrays(A, PG_POS_F32, src->n, dst->nvar) != PG_OK)
+      if (alloc_arrays(A, PG_POS_F32, src->n, dst->nvar, uses ? 0 : src->n) != PG_OK)
         return cudaErrorMemoryAllocation;
       pset_arrays(dst).free_all();
       pset_set_arrays(dst, A);
@@ -461,9 +464,9 @@ pg_status pg_surrogate_run(pg_pset *ps, pg_mlp *net, const pg_kernel *k, int nst
     // packed into a dense set
     if (h_nrej > 0) {
       const int64_t m = (int64_t)h_nrej;
-      if (rset->cap < m) {
+      if (rset->cap < m || (uses && rset->n == 0)) {
         PsetArrays A;
-        if (alloc_arrays(A, PG_POS_F32, m, rset->nvar) != PG_OK) {
+        if (alloc_arrays(A, PG_POS_F32, m, rset->nvar, uses ? 0 : m) != PG_OK) {
           r = PG_ERR_NOMEM;
           set_error("surrogate fallback set of %lld particles", (long long)m);
           break;
